@@ -251,6 +251,10 @@ struct fusion_model {
     bool fp8 = false;             // conv operands in FP8 E4M3 (per-channel weight, per-pose activation scales)
     size_t esz = 4;               // bytes per grid / activation element
     ConvTcPlan tcplan[FUSION_MAX_CONV];
+    // FP32 path: layers on the tensor cores as two-part FP16 products (the others on the CUDA cores)
+    bool f32tc[FUSION_MAX_CONV] = {};
+    ConvF32TcPlan f32plan[FUSION_MAX_CONV];
+    int f32_fold = -1;                            // first layer reads its input x-folded at this pad, or -1
     DenseTcPlan dense_tc;                         // tensor-core CNN dense (bf16 / FP8 models)
     int dense_tc_splits = 0;
     int pool_n = 0, pool_c = 0, flat = 0, splits = 1;
@@ -275,9 +279,9 @@ struct fusion_model {
     int fp8_fold = -1;                            // FP8: first conv reads the folded FP8 grid (this pad), or -1
     void *act[FUSION_MAX_CONV] = {};
     void *pool_out = nullptr;
-    void *qbuf = nullptr;         // FP8 input of the conv layer being computed
-    float *amax = nullptr, *qscale = nullptr;   // FP8: per-pose max |activation| and scale [max_poses]
-    float *conv_sw[FUSION_MAX_CONV] = {};       // FP8: per-output-channel weight scales
+    void *qbuf = nullptr;         // FP8 input (FP32: the input's two FP16 parts) of the conv layer being computed
+    float *amax = nullptr, *qscale = nullptr;   // per-pose max |activation| and scale (FP32: its inverse) [max_poses]
+    float *conv_sw[FUSION_MAX_CONV] = {};       // per-output-channel weight scales (FP32: their inverses)
     float *dense_part = nullptr, *cnn_lat = nullptr;
     float *cnn_lat2 = nullptr;    // second CNN dense layer's output (the CNN latent when present)
     int32_t *e_beg[2] = {}, *e_deg[2] = {}, *e_col[2] = {};
@@ -438,6 +442,53 @@ std::vector<float> pad_vec(const float *b, int n, int N, int groups = 1) {   // 
         if (rc_) return rc_;  \
     } while (0)
 
+// Layout of the FP16 parts an FP32 layer reads: channel-blocked at stride 1, parity-split at stride 2 where the
+// size is even, else NDHWC.
+int f32tc_layout(const fusion_model *m, int i) {
+    return m->d.conv[i].stride == 1 ? 1 : m->conv[i].n_in % 2 == 0 ? 2 : 0;
+}
+int f32tc_channels(const fusion_model *m, int i) { return i == 0 ? 32 : m->d.conv[i].c_in; }   // 19 padded to 32
+
+// The tensor-core weights and plan of FP32 layer i, on success in m->f32tc[i] (else the layer stays on the CUDA
+// cores: a kernel size no tile fits, or no room for the parts).
+int plan_f32tc(fusion_model *m, int i, const float *w, float *bias) {
+    const fusion_conv_desc &c = m->d.conv[i];
+    const int nt = conv_f32tc_block(c.c_out);
+    if (!m->qbuf || !nt) return FUSION_OK;
+    const int cp = f32tc_channels(m, i), fold = i == 0 && m->f32_fold >= 0 ? 1 : 0;
+    const size_t bytes = conv_tc_weight_bytes(cp, nt, c.k, c.stride, 2, fold) * (c.c_out / nt);
+    std::vector<uint8_t> hi(bytes), both(2 * bytes);
+    std::vector<float> isw(c.c_out);
+    conv_f32tc_arrange_weights(w, c.c_out, c.c_in, cp, c.k, c.stride, fold, hi.data(), both.data(), isw.data());
+    void *d_hi = nullptr, *d_both = nullptr;
+    RC_INNER(upload_raw(m, &d_hi, hi.data(), bytes));
+    RC_INNER(upload_raw(m, &d_both, both.data(), 2 * bytes));
+    RC_INNER(upload(m, &m->conv_sw[i], isw));
+    ConvF32TcSpec sp{};
+    sp.x = m->qbuf;
+    sp.max_poses = m->d.max_poses;
+    sp.n_in = m->conv[i].n_in;
+    sp.cin_pad = cp;
+    sp.w_hi = d_hi;
+    sp.w_both = d_both;
+    sp.inv_sw = m->conv_sw[i];
+    sp.inv_sx = m->qscale;
+    sp.bias = bias;
+    sp.xres = i > 0 ? static_cast<const float *>(m->act[i - 1]) : nullptr;
+    sp.y = static_cast<float *>(m->act[i]);
+    sp.n_out = m->conv[i].n_out;
+    sp.c_out = c.c_out;
+    sp.k = c.k;
+    sp.stride = c.stride;
+    sp.residual = c.residual;
+    sp.err = m->err;
+    sp.fold = fold;
+    sp.blocked = f32tc_layout(m, i);
+    char why[256] = {0};
+    m->f32tc[i] = conv_f32tc_plan(m->f32plan[i], sp, why, sizeof(why)) == 0;
+    return FUSION_OK;
+}
+
 int load_weights(fusion_model *m, const float *blob) {
     const fusion_model_desc &d = m->d;
     const std::vector<TensorSpec> L = blob_layout(d);
@@ -468,7 +519,11 @@ int load_weights(fusion_model *m, const float *blob) {
             conv_tc_arrange_weights(w, c.c_out, c.c_in, cx, c.k, c.stride, elem, fold, t.data(), sw.data());
             RC(upload_raw(m, &m->conv[i].w, t.data(), t.size()));
             if (m->fp8) RC(upload(m, &m->conv_sw[i], sw));
-        } else {
+        }
+        RC(upload(m, &m->conv[i].b, std::vector<float>(b, b + c.c_out)));
+        m->conv[i].cx_in = cx;
+        if (!m->bf16) RC(plan_f32tc(m, i, w, m->conv[i].b));
+        if (!m->bf16 && !m->f32tc[i]) {
             std::vector<float> t((size_t)k3 * cx * c.c_out, 0.f);
             for (int o = 0; o < c.c_out; ++o)
                 for (int ci = 0; ci < c.c_in; ++ci)
@@ -476,8 +531,6 @@ int load_weights(fusion_model *m, const float *blob) {
                         t[((size_t)q * cx + ci) * c.c_out + o] = w[((size_t)o * c.c_in + ci) * k3 + q];
             RC(upload_raw(m, &m->conv[i].w, t.data(), t.size() * 4));
         }
-        RC(upload(m, &m->conv[i].b, std::vector<float>(b, b + c.c_out)));
-        m->conv[i].cx_in = cx;
     }
     // dense: input index c*S^3 + sp  ->  sp*C + c
     {
@@ -637,6 +690,17 @@ int alloc_workspace(fusion_model *m) {
         RC(dalloc_bytes(m, &m->qbuf, qmax));
         RC(dalloc(m, &m->amax, B));
         RC(dalloc(m, &m->qscale, B));
+    }
+    if (!m->bf16) {
+        // the largest layer input as two FP16 parts; without room for it the layers stay on the CUDA cores
+        size_t parts = 0;
+        for (int i = 0; i < d.n_conv; ++i) {
+            const size_t n = conv_out(d, i).n;
+            parts = std::max(parts, B * n * n * n * f32tc_channels(m, i) * 4);
+        }
+        RC(dalloc(m, &m->amax, B));
+        RC(dalloc(m, &m->qscale, B));
+        if (dalloc_bytes(m, &m->qbuf, parts) != FUSION_OK) m->qbuf = nullptr;
     }
     if (m->bf16) m->dense_tc_splits = dense_tc_splits(m->flat, d.cnn_dense);
     RC(dalloc(m, &m->dense_part, std::max((size_t)std::max(m->splits, m->dense_tc_splits) * B * d.cnn_dense,
@@ -878,6 +942,8 @@ int fusion_create(const fusion_model_desc *desc, const void *weights, size_t wei
         // (4 + 1 x-offsets per kernel row instead of 7 for one 32-channel chunk 13/32 zero)
         if (m->fp8 && !c0.residual && conv_tc_fold_ok(c0.c_in, m->grid_cx, c0.k, c0.stride, 1))
             m->fp8_fold = c0.k / 2;
+        // FP32 on the tensor cores: the first layer's FP16 parts are folded as the BF16 grid is
+        if (!m->bf16 && !c0.residual && conv_tc_fold_ok(c0.c_in, 32, c0.k, c0.stride, 2)) m->f32_fold = c0.k / 2;
     }
     int rc = alloc_workspace(m);
     if (!rc) rc = load_weights(m, static_cast<const float *>(weights));
@@ -1063,9 +1129,9 @@ static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, 
     };
     VoxArgs va{off_d, B, d.grid_n, d.support, d.max_atoms, m->grid, m->grid_cx,
                m->bf16 ? 1 : 0, m->grid_fold, bf16_blocked_in(m, 0) ? 1 : 0, m->cell_row, m->atom_rec,
-               m->fp8 ? m->amax : nullptr};
-    // FP8: voxelize also reduces each pose's max |grid value| (the first layer's input scale)
-    if (m->fp8) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
+               m->fp8 || m->f32tc[0] ? m->amax : nullptr};
+    // FP8 and FP32: voxelize also reduces each pose's max |grid value| (the first layer's input scale)
+    if (va.amax) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
     launch_voxelize(va, st);
     RC(check_launch("voxelize"));
     map[1] = ei; mark(st);
@@ -1085,6 +1151,19 @@ static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, 
             conv_tc_launch(m->tcplan[i], B, st);
         } else if (m->bf16) {
             conv_tc_launch(m->tcplan[i], B, st);
+        } else if (m->f32tc[i]) {
+            const size_t n = m->conv[i].n_in;
+            if (i > 0 && !m->f32tc[i - 1]) {       // the CUDA-core layer before left no maximum
+                CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
+                launch_amax_f32(static_cast<const float *>(x), B, n * n * n * m->conv[i].cx_in, m->amax, st);
+            }
+            SplitF16Args sa{static_cast<const float *>(x), static_cast<__half *>(m->qbuf), (int)n, m->conv[i].cx_in,
+                            f32tc_channels(m, i), d.max_poses, f32tc_layout(m, i), i == 0 ? m->f32_fold : -1, m->amax,
+                            m->qscale};
+            launch_split_f16(sa, B, st);
+            const bool next = i + 1 < d.n_conv && m->f32tc[i + 1];
+            if (next) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
+            conv_f32tc_launch(m->f32plan[i], B, next ? m->amax : nullptr, st);
         } else {
             ConvArgs ca{static_cast<const float *>(x), static_cast<const float *>(m->conv[i].w), m->conv[i].b,
                         static_cast<float *>(m->act[i]), B, m->conv[i].n_in, m->conv[i].n_out,
@@ -1472,7 +1551,7 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value) {
         if (value != 1 && value != 2) return fail(FUSION_EINVAL, "the wait-timeout test takes value 1 or 2");
         if (m->use_graph) return fail(FUSION_EUNSUPPORTED, "turn CUDA graphs off for the wait-timeout test");
         if (value == 1) {
-            if (!m->bf16) return fail(FUSION_EUNSUPPORTED, "the FP32 path has no bounded tensor-core waits");
+            if (!m->bf16) return fail(FUSION_EUNSUPPORTED, "the conv wait-timeout test needs a BF16 or FP8 model");
             conv_tc_stall_next(m->tcplan[0]);
         } else {
             if (!m->sg_tc) return fail(FUSION_EUNSUPPORTED, "the graph convolution is not on the tensor cores");

@@ -8,6 +8,7 @@
 
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "../../include/fusion.h"
@@ -67,7 +68,7 @@ struct VoxArgs {
     int blocked;          // bf16 only: store channel-blocked, [B][n][n][cx / 8][n][8]
     const int32_t *cell_row;     // PrepArgs::cell_row
     const float *atom_rec;       // PrepArgs::atom_rec (records in cell order)
-    float *amax;          // bf16 only, may be null: per-pose max |stored value| (atomic max; zeroed by the caller)
+    float *amax;          // cx 24 or 32, may be null: per-pose max |stored value| (atomic max; zeroed by the caller)
 };
 void launch_voxelize(const VoxArgs &a, cudaStream_t s);
 
@@ -178,6 +179,59 @@ void conv_tc_launch(ConvTcPlan &plan, int B, cudaStream_t s);
 // and it sets FUSION_ERR_TIMEOUT; later launches are normal.
 void conv_tc_stall_next(ConvTcPlan &plan);
 void conv_tc_describe(const ConvTcPlan &plan, int *T, int *groups_per_stage, int *nbs, size_t *smem, int *group);
+
+// x-offsets of the two chunks of an x-folded first layer (mode 1 bf16 / f16 grid, 2 FP8 grid): chunk c is read
+// at n[c] offsets start[c] + step[c] * t.
+void conv_tc_fold_pattern(int mode, int k, int n[2], int step[2], int start[2]);
+
+// FP32 conv on the tensor cores (k_conv_f32tc.cu): x and w as two FP16 parts each, three products.
+struct ConvF32TcPlan {
+    struct Impl;
+    Impl *impl;
+    ConvF32TcPlan();
+    ~ConvF32TcPlan();
+    ConvF32TcPlan(const ConvF32TcPlan &) = delete;
+    ConvF32TcPlan &operator=(const ConvF32TcPlan &) = delete;
+};
+struct ConvF32TcSpec {
+    const void *x;          // the input's FP16 parts (launch_split_f16): [2][max_poses] maps of cin_pad channels
+    int max_poses, n_in, cin_pad;
+    const void *w_hi, *w_both;   // arranged weights (conv_f32tc_arrange_weights)
+    const float *inv_sw;    // [c_out] 1 / weight scale
+    const float *inv_sx;    // [max_poses] 1 / input scale
+    const float *bias;      // [c_out]
+    const float *xres;      // residual source [max_poses][n_in]^3[c_out]
+    float *y;               // [max_poses][n_out]^3[c_out], NDHWC
+    int n_out, c_out, k, stride, residual;
+    unsigned *err;
+    int fold;               // 1: x-folded first-layer input (launch_split_f16 with fold_pad = k / 2)
+    int blocked;            // layout of the parts: 0 NDHWC, 1 channel-blocked, 2 parity-split (ConvTcSpec::blocked)
+};
+// 0, or nonzero with a reason: the caller then uses launch_conv3d_f32.
+int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &spec, char *why, size_t why_len);
+// amax: per-pose max |output| (atomic max, zeroed by the caller), or null.
+void conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s);
+// Output channels per tile (0: c_out is not a multiple of 32).
+int conv_f32tc_block(int c_out);
+// Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two; inv_sw[co] = 1 / s_w[co].  Per block of
+// NT = conv_f32tc_block(c_out) output channels, in the layout of conv_tc_arrange_weights (elem 2) for NT channels:
+// w_hi has rows [tz][hi of NT channels], w_both rows [tz][hi of NT channels, lo of NT channels].  w_hi takes
+// c_out / NT x conv_tc_weight_bytes(cin_pad, NT, k, stride, 2, fold) bytes, w_both twice that.
+void conv_f32tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad, int k, int stride, int fold,
+                                uint8_t *w_hi, uint8_t *w_both, float *inv_sw);
+// The two FP16 parts of B poses' FP32 NDHWC maps (x * 2^e = hi + lo, 2^e per pose from amax).
+struct SplitF16Args {
+    const float *x;         // [B][n]^3[c], c a multiple of 8
+    __half *out;            // [2][max_poses][n^3 cp]: high parts, then low parts
+    int n, c, cp, max_poses;
+    int layout;             // 0 NDHWC, 1 channel-blocked, 2 parity-split
+    int fold_pad;           // >= 0 (cp = 32, layout 1): channels 16..18 folded along x as in VoxArgs::fold_pad
+    const float *amax;      // [B] max |x| of each pose
+    float *inv_sx;          // [B] 2^-e
+};
+void launch_split_f16(const SplitF16Args &a, int B, cudaStream_t s);
+// Per-pose max |x| of FP32 maps (atomic max, zeroed by the caller); per_pose a multiple of 4.
+void launch_amax_f32(const float *x, int B, size_t per_pose, float *amax, cudaStream_t s);
 
 // Per-pose FP8 quantization of the plain bf16 grid [B][n]^3[32] (channels 0..18) into the folded layout
 // the first FP8 conv reads, [B][n][n][n + 1][64]: stored voxel j holds channels 0..15 of grid voxels

@@ -96,6 +96,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <vector>
 
 namespace fusion {
 
@@ -619,7 +620,7 @@ bool conv_tc_fold_ok(int c_in, int cin_pad, int k, int stride, int elem) {
     return stride == 1 && (k == 3 || k == 5 || k == 7) && c_in == 19 && cin_pad == 32 && (elem == 1 || elem == 2);
 }
 
-static void fold_pattern(int mode, int k, int n[2], int step[2], int start[2]) {
+void conv_tc_fold_pattern(int mode, int k, int n[2], int step[2], int start[2]) {
     const int p = k / 2;
     if (mode == 1) {
         n[0] = k; step[0] = 1; start[0] = 0;
@@ -635,7 +636,7 @@ size_t conv_tc_weight_bytes(int cin_pad, int c_out, int k, int stride, int elem,
     const int chunks = cin_pad * elem / chunk_bytes_in;
     if (!fold) return (size_t)chunks * chunk_weight_bytes(c_out, k, stride);
     int n[2], st[2], s0[2];
-    fold_pattern(fold, k, n, st, s0);
+    conv_tc_fold_pattern(fold, k, n, st, s0);
     return (size_t)k * (n[0] + n[1]) * k * 2 * c_out * 16;
 }
 
@@ -672,35 +673,16 @@ static uint16_t bf16_from_float(float v) {
     return (uint16_t)(u >> 16);
 }
 
-void conv_tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad, int k, int stride, int elem,
-                             int fold, uint8_t *out, float *s_w) {
-    // blob layout w[co][ci][kd][kh][kw] ->
-    //   [chunk][phase][ty][tx][8/16-channel half][tz = nz-1 .. 0][co][16 bytes]
-    const int cpr = elem == 2 ? 8 : 16;                // channels per 16-byte row
+// Walks blob weights w[co][ci][kd][kh][kw] in the arranged order, calling put(value, co) per 16-byte-row element:
+//   [chunk][phase][ty][tx][cpr-channel half][tz = nz-1 .. 0][co][16 bytes], cpr channels per 16-byte row
+template <class Put>
+static void walk_weights(const float *w, int c_out, int c_in, int cin_pad, int k, int stride, int cpr, int fold, Put put) {
     const int nph = stride == 1 ? 1 : 8;
-    const int k3 = k * k * k;
-    if (elem == 1) {
-        for (int co = 0; co < c_out; ++co) {
-            float mx = 0.f;
-            for (int q = 0; q < c_in * k3; ++q) mx = std::fmax(mx, std::fabs(w[(size_t)co * c_in * k3 + q]));
-            s_w[co] = mx > 0.f ? mx / 448.f : 1.f;
-        }
-    }
-    size_t idx = 0;
-    auto put = [&](float v, int co) {
-        if (elem == 2) {
-            const uint16_t h = bf16_from_float(v);
-            memcpy(out + idx, &h, 2);
-            idx += 2;
-        } else {
-            out[idx++] = e4m3_from_float(v / s_w[co]);
-        }
-    };
     if (fold) {
         // folded first-layer input: two chunks of 2 x cpr slots; slot q of chunk c at x-offset t reads
         // channel ch and kernel column kw, or nothing
         int nt[2], st[2], s0[2];
-        fold_pattern(fold, k, nt, st, s0);
+        conv_tc_fold_pattern(fold, k, nt, st, s0);
         for (int c = 0; c < 2; ++c)
             for (int ty = 0; ty < k; ++ty)
                 for (int t = 0; t < nt[c]; ++t)
@@ -738,19 +720,68 @@ void conv_tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad, i
                             for (int co = 0; co < c_out; ++co)
                                 for (int el = 0; el < cpr; ++el) {
                                     const int ci = c * 2 * cpr + half * cpr + el;
-                                    float v = 0.f;
-                                    if (ci < c_in) v = w[((((size_t)co * c_in + ci) * k + kd) * k + kh) * k + kw];
-                                    if (elem == 2) {
-                                        const uint16_t h = bf16_from_float(v);
-                                        memcpy(out + idx, &h, 2);
-                                        idx += 2;
-                                    } else {
-                                        out[idx++] = e4m3_from_float(v / s_w[co]);
-                                    }
+                                    put(ci < c_in ? w[((((size_t)co * c_in + ci) * k + kd) * k + kh) * k + kw] : 0.f, co);
                                 }
                         }
         }
     }
+}
+
+// max |w| of output channel co.
+static float channel_max(const float *w, int co, size_t per) {
+    float mx = 0.f;
+    for (size_t q = 0; q < per; ++q) mx = std::fmax(mx, std::fabs(w[(size_t)co * per + q]));
+    return mx;
+}
+
+void conv_tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad, int k, int stride, int elem,
+                             int fold, uint8_t *out, float *s_w) {
+    const size_t per = (size_t)c_in * k * k * k;
+    if (elem == 1)
+        for (int co = 0; co < c_out; ++co) {
+            const float mx = channel_max(w, co, per);
+            s_w[co] = mx > 0.f ? mx / 448.f : 1.f;
+        }
+    size_t idx = 0;
+    walk_weights(w, c_out, c_in, cin_pad, k, stride, elem == 2 ? 8 : 16, fold, [&](float v, int co) {
+        if (elem == 2) {
+            const uint16_t h = bf16_from_float(v);
+            memcpy(out + idx, &h, 2);
+            idx += 2;
+        } else {
+            out[idx++] = e4m3_from_float(v / s_w[co]);
+        }
+    });
+}
+
+void conv_f32tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad, int k, int stride, int fold,
+                                uint8_t *w_hi, uint8_t *w_both, float *inv_sw) {
+    const size_t per = (size_t)c_in * k * k * k;
+    const int NT = conv_f32tc_block(c_out);
+    std::vector<float> s(c_out);
+    for (int co = 0; co < c_out; ++co) {
+        // 2^e puts the channel's largest weight in [2^14, 2^15)
+        const float mx = channel_max(w, co, per);
+        int e = 0;
+        if (mx > 0.f && std::isfinite(mx)) e = 14 - std::ilogb(mx);
+        if (e > 126) e = 126;
+        s[co] = std::ldexp(1.f, e);
+        inv_sw[co] = std::ldexp(1.f, -e);
+    }
+    size_t idx = 0;                              // elements of w_hi so far
+    for (int c0 = 0; c0 < c_out; c0 += NT)
+        walk_weights(w + (size_t)c0 * per, NT, c_in, cin_pad, k, stride, 8, fold, [&](float v, int co) {
+            const float t = v * s[c0 + co];      // exact: a power of two
+            const __half h = __float2half_rn(t);
+            const float r = t - __half2float(h);
+            const __half l = __float2half_rn(std::isfinite(r) ? r : 0.f);
+            const size_t run = (size_t)NT * 8;   // elements of one offset's NT rows
+            const size_t both = idx / run * 2 * run + idx % run;
+            memcpy(w_hi + 2 * idx, &h, 2);
+            memcpy(w_both + 2 * both, &h, 2);
+            memcpy(w_both + 2 * (both + run), &l, 2);
+            ++idx;
+        });
 }
 
 int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_len) {
@@ -928,7 +959,7 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
     A.residual = sp.residual;
     A.xpat = sp.fold ? 1 : 0;
     A.x_shift = sp.fold == 2 ? 1 : 0;
-    if (sp.fold) fold_pattern(sp.fold, k, A.xt_n, A.xt_step, A.xt_start);
+    if (sp.fold) conv_tc_fold_pattern(sp.fold, k, A.xt_n, A.xt_step, A.xt_start);
     A.blocked = sp.blocked;
     A.out_blocked = sp.out_blocked;
     A.res_blocked = sp.res_blocked;

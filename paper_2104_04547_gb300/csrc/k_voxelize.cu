@@ -232,7 +232,7 @@ __device__ __forceinline__ size_t bf16_block_off(int p, int z, int y, int x, int
 
 // BPW: x-boxes per warp (a tile spans whole x-rows: ceil(n / 4) boxes; warp w takes boxes w, w + 6, ..., so
 // each warp holds boxes from both halves of the row and the warps' work evens out).
-// AMAX: also reduce the pose's max |stored value| (the FP8 path's first input scale).
+// AMAX: also reduce the pose's max |stored value| (the first layer's input scale of the FP8 and FP32 paths).
 template <bool BF16, int CX, bool AMAX, int BPW>
 __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
         __syncthreads();
     }
 
-    float vmax = 0.f;                                  // max |stored bf16 value| of this thread's voxels
+    float vmax = 0.f;                                  // max |stored value| of this thread's voxels
     const bool fold = BF16 && a.fold_pad >= 0;
     const int W = nxb * 4;
 #pragma unroll 1
@@ -433,6 +433,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
                     v4.z = c0 + 2 < kFeat ? acc[c0 + 2 < kFeat ? c0 + 2 : 0] : 0.f;
                     v4.w = c0 + 3 < kFeat ? acc[c0 + 3 < kFeat ? c0 + 3 : 0] : 0.f;
                     *reinterpret_cast<float4 *>(out + c0) = v4;
+                    if (AMAX) vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(v4.x), fabsf(v4.y))), fmaxf(fabsf(v4.z), fabsf(v4.w)));
                 }
             }
         }
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
         }
     }
     if constexpr (AMAX) {
-        // the pose's max |grid value| for the FP8 input scale: warps, then one atomic per CTA
+        // the pose's max |grid value| for the first layer's input scale: warps, then one atomic per CTA
         __shared__ float s_wmax[kVoxWarps];
         for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
         if (lane == 0) s_wmax[warp] = vmax;
@@ -527,7 +528,8 @@ void launch_voxelize(const VoxArgs &a, cudaStream_t s) {
         if (a.amax) launch_vox_p<true, 32, true>(a, s);
         else launch_vox_p<true, 32, false>(a, s);
     } else if (a.cx == 24) {
-        launch_vox_p<false, 24, false>(a, s);
+        if (a.amax) launch_vox_p<false, 24, true>(a, s);
+        else launch_vox_p<false, 24, false>(a, s);
     } else {
         launch_vox_p<false, 20, false>(a, s);
     }

@@ -71,10 +71,9 @@
 // each further one from a global counter, passing the index on to the other
 // roles through a small ring in shared memory.  Roles: warp 0 lane 0 issues the TMA
 // loads, running ahead into the next tile while the current one finishes;
-// warp 1 owns tensor memory; lane 0 of warps 1..NI issues the MMAs of its share
-// of the slice groups (one issuing thread was measured to limit the MMA rate,
-// so several warps issue; each commits its own MMAs and the empty barriers
-// count NI arrivals); the remaining 4 x EPW warps run the epilogue (tensor
+// warp 1 owns tensor memory; warps 1..NI issue the MMAs of their share of the
+// slice groups, converged with one elected lane issuing (see issue_groups; each
+// commits its own MMAs and the empty barriers count NI arrivals); the remaining 4 x EPW warps run the epilogue (tensor
 // memory -> registers, bias, ReLU, residual add, bf16 stores in NDHWC or
 // channel-blocked order), EPW per
 // tensor-memory lane quarter (a warp reaches only the lanes of quarter
@@ -103,6 +102,7 @@ namespace fusion {
 namespace {
 
 constexpr int kIssReq = 4;
+constexpr int kMaxHalos = 4; // halo buffers at most
 constexpr int kRing = 4;     // tile indices the producer publishes ahead of the issuers and the epilogue
 
 // Warp roles of one kernel instance: warp 0 loads, warps 1..NI issue MMAs, then 4 x EPW epilogue warps
@@ -174,13 +174,45 @@ __device__ __forceinline__ void phase_taps(const Args &a, int ph, int &pz, int &
     }
 }
 
+// The MMAs of `cnt` (ty, tx) groups into DPI slice groups, from column tx: plane u of a group feeds its slices
+// s_lo..s_hi (offset tz = u - s) in one MMA.  NZ is a template parameter so that a group's MMAs unroll: widths,
+// accumulator columns and weight rows become constants and an MMA costs one add.  With these computed in a runtime
+// loop under a one-lane branch (166 to 210 clocks per MMA and issuing warp, against 45 here, with constant operands)
+// the issuing warps' scalar work, not the tensor pipe, set the pace of every layer whose MMAs are narrow.  Measured at
+// 64 poses: paper-final 48^3 residual layer 1174 -> 1036 us BF16, its stride-2 layer 217 -> 197 us; full-size stride-2
+// layer 1422 -> 1230 us; full-size residual layers, whose MMAs are wide, 9.43 -> 9.31 ms.
+template <int NZ, int N, int G, int DPI, bool F8>
+__device__ __forceinline__ void issue_groups(uint32_t on, uint32_t dt, uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh,
+                                             int cnt, int tx, int nx, int xstep, uint32_t wrap, uint32_t row_zy) {
+    constexpr uint32_t IDESC0 = (F8 ? tc::idesc_e4m3(128, 8) : tc::idesc_bf16(128, 8)) & ~(0x3Fu << 17);
+#pragma unroll 1
+    for (int i = 0; i < cnt; ++i) {
+        uint32_t ad[DPI];
+#pragma unroll
+        for (int dd = 0; dd < DPI; ++dd) ad[dd] = al + (uint32_t)(G * dd) * row_zy;
+#pragma unroll
+        for (int u = 0; u <= NZ + G - 2; ++u) {
+            const int s_lo = u > NZ - 1 ? u - (NZ - 1) : 0;
+            const int s_hi = u < G - 1 ? u : G - 1;
+            const uint32_t idesc = IDESC0 | ((uint32_t)((s_hi - s_lo + 1) * N) >> 3) << 17;
+#pragma unroll
+            for (int dd = 0; dd < DPI; ++dd) {
+                tc::mma_acc<F8>(on, dt + (uint32_t)((G * dd + s_lo) * N), ad[dd], ah,
+                                bl + (uint32_t)((NZ - 1 - (u - s_lo)) * N), bh, idesc);
+                ad[dd] += row_zy;
+            }
+        }
+        bl += (uint32_t)(NZ * N * 2);   // next group: NZ * N * 32 bytes
+        if (++tx == nx) { tx = 0; al += wrap; }
+        else al += (uint32_t)xstep;
+    }
+}
+
 template <int N, int T, bool F8, int G>
 __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(const __grid_constant__ CUtensorMap tmap, Args a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     static_assert(T % G == 0 && G * N <= 256, "a slice group divides T and spans at most 256 columns");
     constexpr uint32_t TCOLS = (T * N <= 32) ? 32 : (T * N <= 64) ? 64 : (T * N <= 128) ? 128 : (T * N <= 256) ? 256 : 512;
-    // instruction descriptor without its N field (bits 17..22 = N / 8, set per MMA)
-    constexpr uint32_t IDESC0 = (F8 ? tc::idesc_e4m3(128, 8) : tc::idesc_bf16(128, 8)) & ~(0x3Fu << 17);
     using R = Roles<N, T, G>;
     constexpr int UNITS = R::UNITS, NI = R::NI, UCOLS = R::UCOLS, EPW = R::EPW, PART = R::PART, EPI0 = R::EPI0;
     constexpr int DPI = UNITS / NI;
@@ -191,9 +223,9 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     unsigned char *sA = smem;
     unsigned char *sB = smem + g.na * a_bytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(sB + g.nbs * g.stage_bytes);
-    uint64_t *a_full = bars;            // [2]
-    uint64_t *a_empty = bars + 2;       // [2]
-    uint64_t *b_full = bars + 4;        // [nbs]
+    uint64_t *a_full = bars;            // [na]
+    uint64_t *a_empty = bars + g.na;    // [na]
+    uint64_t *b_full = a_empty + g.na;  // [nbs]
     uint64_t *b_empty = b_full + g.nbs; // [nbs]
     uint64_t *acc_full = b_empty + g.nbs;   // [UNITS]: the tile's MMAs of the group are complete
     uint64_t *acc_empty = acc_full + UNITS; // [UNITS]: the epilogue has read and re-zeroed the group
@@ -204,7 +236,8 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tile_ring + kRing);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // the shuffle tells the compiler that the warp index is uniform
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int n_tiles = g.nbx * g.nby * g.nbz * a.B;
     auto decode = [&](int t, int &x0, int &y0, int &z0, int &b) {
         x0 = (t % g.nbx) * 8; t /= g.nbx;
@@ -214,7 +247,7 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     };
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) { tc::mbar_init(&a_full[i], 1); tc::mbar_init(&a_empty[i], NI); }
+        for (int i = 0; i < g.na; ++i) { tc::mbar_init(&a_full[i], 1); tc::mbar_init(&a_empty[i], NI); }
         for (int i = 0; i < g.nbs; ++i) { tc::mbar_init(&b_full[i], 1); tc::mbar_init(&b_empty[i], NI); }
         for (int u = 0; u < UNITS; ++u) { tc::mbar_init(&acc_full[u], 1); tc::mbar_init(&acc_empty[u], 4 * EPW); }
         tc::mbar_init(mma_done, NI);
@@ -305,31 +338,38 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
             }
             tile = atomicAdd(a.tile_counter, 1) + (int)gridDim.x;
         }
-    } else if (warp >= 1 && warp <= NI && lane == 0) {
-        const int d0 = (warp - 1) * DPI;
+    } else if (warp >= 1 && warp <= NI) {
         // ---------------- MMA issuer ----------------
-        int ai = 0, bi = 0;
+        // All lanes run the loops, so that the MMAs' operands sit in uniform registers; one elected lane issues.
+        const int d0 = (warp - 1) * DPI;
+        const uint32_t on = tc::elect_one();
+        auto wait_all = [&](uint64_t *bar, uint32_t parity, uint64_t deadline) {
+            return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, deadline, a.err, FUSION_ERR_TIMEOUT)) != 0;
+        };
+        int ai = 0, st = 0;                 // halo buffers so far; weight stage in turn and its parity
+        uint32_t b_par = 0;
         const uint32_t sbo_a = (uint32_t)g.ystep * 16;
         const uint32_t row_zy = (uint32_t)g.hh * g.ystep;
+        const uint32_t dt = tbase + (uint32_t)(G * d0 * N);
         for (int it = 0;; ++it) {
             const uint64_t deadline = tc::globaltimer() + kWaitNs;
             const int slot = it % kRing;
-            if (!tc::mbar_wait(&tile_full[slot], (it / kRing) & 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
-            const int tile = tile_ring[slot];
-            tc::mbar_arrive(&tile_empty[slot]);
-            if (tile < 0 || *abort_flag) break;
+            if (!wait_all(&tile_full[slot], (it / kRing) & 1, deadline)) { fail(); break; }
+            const bool done = __any_sync(0xffffffffu, tile_ring[slot] < 0 || *abort_flag != 0);   // every lane has read the slot
+            if (on) tc::mbar_arrive(&tile_empty[slot]);
+            if (done) break;
             // this warp's slice groups must have been read (and re-zeroed) by the previous tile's epilogue
             bool ok = true;
-            for (int dd = 0; dd < DPI && ok; ++dd)
-                ok = tc::mbar_wait(&acc_empty[d0 + dd], (it & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT);
+            for (int dd = 0; dd < DPI && ok; ++dd) ok = wait_all(&acc_empty[d0 + dd], (it & 1) ^ 1, deadline);
             if (!ok) { fail(); break; }
             tc::tc_fence_after();
-            for (int c = 0; c < g.chunks && !*abort_flag; ++c) {
-                for (int ph = 0; ph < g.nphase && !*abort_flag; ++ph) {
+            for (int c = 0; c < g.chunks && ok; ++c) {
+                for (int ph = 0; ph < g.nphase && ok; ++ph) {
                     int pz, py, px, nz, ny, nx;
                     phase_taps(a, ph, pz, py, px, nz, ny, nx);
                     const int buf = ai % g.na;
-                    if (!tc::mbar_wait(&a_full[buf], (ai / g.na) & 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
+                    ok = wait_all(&a_full[buf], (ai / g.na) & 1, deadline);
+                    if (!ok) { fail(); break; }
                     // descriptors advance by plain integer adds: the start-address field counts 16-byte rows
                     const uint64_t adesc0 = tc::desc_kmajor(tc::smem_u32(sA + buf * a_bytes), g.lbo_a, sbo_a);
                     const uint32_t lbo_b = (uint32_t)nz * N * 16;    // between the two 8-channel halves
@@ -341,43 +381,42 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                         xstart = a.xt_start[c];
                     }
                     const int ngr = nz > 0 ? ny * nx : 0;   // a phase without z taps adds nothing
-                    for (int g0 = 0; g0 < ngr; g0 += g.groups_per_stage) {
-                        const int gend = min(g0 + g.groups_per_stage, ngr);
-                        const int st = bi % g.nbs;
-                        if (!tc::mbar_wait(&b_full[st], (bi / g.nbs) & 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
+                    const uint32_t ah = (uint32_t)(adesc0 >> 32), wrap = (uint32_t)(g.ystep - xstep * (nx - 1));
+                    uint32_t al = (uint32_t)adesc0 + (uint32_t)xstart + (uint32_t)(G * d0) * row_zy;
+                    int tx = 0;
+                    for (int g0 = 0; g0 < ngr && ok; g0 += g.groups_per_stage) {
+                        const int cnt = min(g.groups_per_stage, ngr - g0);
+                        ok = wait_all(&b_full[st], b_par, deadline);
+                        if (!ok) { fail(); break; }
                         tc::tc_fence_after();
-                        uint64_t bgrp = tc::desc_kmajor(tc::smem_u32(sB + st * g.stage_bytes), lbo_b, 128);
-                        for (int gi = g0; gi < gend; ++gi) {
-                            const int ty = gi / nx, tx = gi - (gi / nx) * nx;
-                            const int hx = xstart + xstep * tx;
-                            const uint64_t arow = adesc0 + (uint64_t)(ty * g.ystep + hx);
-                            // plane u of slice group j feeds its slices s_lo..s_hi (offset tz = u - s) in one MMA
-                            for (int u = 0; u <= nz + G - 2; ++u) {
-                                const int s_lo = u - (nz - 1) > 0 ? u - (nz - 1) : 0;
-                                const int s_hi = u < G - 1 ? u : G - 1;
-                                const uint32_t idesc = IDESC0 | ((uint32_t)((s_hi - s_lo + 1) * N) >> 3) << 17;
-                                const uint64_t bd = bgrp + (uint64_t)((nz - 1 - (u - s_lo)) * N);
-#pragma unroll
-                                for (int dd = 0; dd < DPI; ++dd) {
-                                    const int j = d0 + dd;
-                                    const uint64_t ad = arow + (uint64_t)((G * j + u) * row_zy);
-                                    const uint32_t dt = tbase + (uint32_t)((G * j + s_lo) * N);
-                                    if constexpr (F8) tc::mma_e4m3(dt, ad, bd, idesc, 1u);
-                                    else tc::mma_bf16(dt, ad, bd, idesc, 1u);
-                                }
-                            }
-                            bgrp += (uint64_t)(nz * N * 2);   // next group: nz * N * 32 bytes
+                        const uint64_t bdesc = tc::desc_kmajor(tc::smem_u32(sB + st * g.stage_bytes), lbo_b, 128);
+                        const uint32_t bl = (uint32_t)bdesc, bh = (uint32_t)(bdesc >> 32);
+                        switch (nz) {     // k and, at stride 2, (k + 1) / 2 and k / 2 for odd k <= 9
+                        case 1: issue_groups<1, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 2: issue_groups<2, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 3: issue_groups<3, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 4: issue_groups<4, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 5: issue_groups<5, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 7: issue_groups<7, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        default: issue_groups<9, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
                         }
-                        tc::mma_commit(&b_empty[st]);
-                        ++bi;
+                        if (on) tc::mma_commit(&b_empty[st]);
+                        for (int i = 0; i < cnt; ++i) {
+                            if (++tx == nx) { tx = 0; al += wrap; }
+                            else al += (uint32_t)xstep;
+                        }
+                        if (++st == g.nbs) { st = 0; b_par ^= 1; }
                     }
-                    tc::mma_commit(&a_empty[buf]);
+                    if (!ok) break;
+                    if (on) tc::mma_commit(&a_empty[buf]);
                     ++ai;
                 }
             }
-            for (int dd = 0; dd < DPI; ++dd) tc::mma_commit(&acc_full[d0 + dd]);
+            if (!ok) break;
+            if (on)
+                for (int dd = 0; dd < DPI; ++dd) tc::mma_commit(&acc_full[d0 + dd]);
         }
-        tc::mma_commit(mma_done);
+        if (on) tc::mma_commit(mma_done);
     } else if (warp >= EPI0) {
         // ---------------- epilogue: EPW warps per tensor-memory lane quarter ----------------
         const int q = warp & 3;                 // lane quarter
@@ -850,14 +889,16 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
         g.lbo_a = g.plane_bytes;
         g.ystep = g.hw;
     }
-    // about 48 KB of weights per stage in a ring of two: each stage hand-off costs a fixed few
-    // hundred cycles, and fewer, larger stages measured faster than deeper rings of smaller ones
+    // about 56 KB of weights per stage in a ring of two (all 9 groups of a 64-channel 3^3 chunk in one stage: 201 ->
+    // 180 us BF16, 182 -> 177 us FP8 for the paper-final 24^3 residual layer at 64 poses, against 8 + 1 groups; the
+    // 7^3 layers take the 3 groups that fit and do not depend on it)
     const uint32_t gbytes_max = (uint32_t)ntmax * c_out * 32;
     // stride 2: about 72 KB per stage, at most one parity phase's groups (a stage never spans phases).  Its
     // small halos leave the room, and fewer weight copies per phase measured faster (full-size conv3, 64
     // poses: 1.47 -> 1.39-1.40 ms BF16, 1.04 -> 1.00-1.01 ms FP8 with 6 groups instead of 4)
-    const uint32_t stage_target = stride == 2 ? 73728u : 49152u;
+    const uint32_t stage_target = stride == 2 ? 73728u : 57344u;
     g.groups_per_stage = sp.groups_per_stage > 0 ? sp.groups_per_stage : (int)(stage_target / gbytes_max);
+    if (sp.groups_per_stage <= 0 && stride == 1 && g.groups_per_stage > ntmax * ntmax) g.groups_per_stage = ntmax * ntmax;
     if (sp.groups_per_stage <= 0 && stride == 2 && g.groups_per_stage > ntmax * ntmax) g.groups_per_stage = ntmax * ntmax;
     if (g.groups_per_stage < 1) g.groups_per_stage = 1;
     g.stage_bytes = ((uint32_t)g.groups_per_stage * gbytes_max + 127) / 128 * 128;
@@ -883,9 +924,9 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
         return -1;
     }
     g.chunks = sp.cin_pad / chunk_ch;
-    // a_full/a_empty [2] each, b_full/b_empty [nbs] each, acc_full/acc_empty [T / group] each, mma_done,
+    // a_full/a_empty [na <= kMaxHalos] each, b_full/b_empty [nbs] each, acc_full/acc_empty [T / group] each, mma_done,
     // tile_full/tile_empty [kRing] each, the tile ring, then the tensor-memory slot and the abort flag
-    const size_t bar_bytes = (size_t)(4 + 2 * g.nbs + 2 * (T / group) + 1 + 2 * kRing) * 8 + kRing * 4 + 16;
+    const size_t bar_bytes = (size_t)(2 * kMaxHalos + 2 * g.nbs + 2 * (T / group) + 1 + 2 * kRing) * 8 + kRing * 4 + 16;
     const size_t limit = 227 * 1024;
     const size_t a1 = g.a_bytes;
     // a larger halo (16 slices per CTA) leaves less room for weights: shrink the default stages to fit
@@ -895,7 +936,11 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
         g.stage_bytes = ((uint32_t)g.groups_per_stage * gbytes_max + 127) / 128 * 128;
     }
     const size_t b_total = (size_t)g.nbs * g.stage_bytes;
-    g.na = (2 * a1 + b_total + bar_bytes <= limit) ? 2 : 1;
+    // as many halo buffers as fit, up to four: at stride 2 the small halos of the parity phases come 8 to a chunk, and
+    // two in flight left the MMAs waiting 30% of the time once these were issued fast enough (paper-final conv2, 64
+    // poses: 197 -> 168 us BF16, 254 -> 244 us FP8)
+    g.na = 1;
+    while (g.na < kMaxHalos && (g.na + 1) * a1 + b_total + bar_bytes <= limit) ++g.na;
     P.smem = g.na * a1 + b_total + bar_bytes;
     if (P.smem > limit) {
         snprintf(why, why_len, "tensor-core conv tile needs %zu bytes of shared memory", P.smem);

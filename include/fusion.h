@@ -279,8 +279,11 @@ int fusion_graph_schedule(fusion_model *m, int32_t *nodes_per_warp);
 
 /* Tile configuration of conv `layer`: out5 = {output slices per CTA, (ty, tx)
  * kernel-offset groups per weight stage, weight stages, shared-memory bytes,
- * adjacent output slices each MMA serves (1, 2 or 4; N = that x output
- * channels)}.  FUSION_EUNSUPPORTED on the FP32 path. */
+ * adjacent output slices each MMA serves (1, 2, 4 or 8; N = that x output
+ * channels)}.  It holds for batches that fill the device; calls whose tiles
+ * would leave multiprocessors idle take fewer slices per CTA (with the same
+ * results), unless FUSION_OPT_CONV_SLICES_PER_MMA fixes the layers' tiles.
+ * FUSION_EUNSUPPORTED on the FP32 path. */
 int fusion_describe_conv(fusion_model *m, int32_t layer, int32_t *out5);
 
 /* ---- aggregation ----

@@ -807,6 +807,7 @@ static ConvTcSpec conv_spec(fusion_model *m, int i) {
     sp.residual = c.residual;
     sp.err = m->err;
     sp.group = m->group_mode;
+    sp.alts = m->group_mode < 0 ? 1 : 0;   // the caller's slices per MMA hold for every launch
     sp.fold = i != 0 ? 0 : m->grid_fold >= 0 ? 1 : m->fp8_fold >= 0 ? 2 : 0;
     if (sp.fold == 2) sp.cin_pad = 64;
     sp.blocked = (fp8_blocked(m, i) || bf16_blocked_in(m, i)) ? 1 : (fp8_split(m, i) || bf16_split_in(m, i, m->split2)) ? 2 : 0;
@@ -1701,7 +1702,9 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
         ConvTcPlan def;
         {
             char why[256] = {0};
-            if (conv_tc_plan(def, conv_spec(m, i), why, sizeof(why))) return fail(FUSION_ECUDA, why);
+            ConvTcSpec sd = conv_spec(m, i);
+            sd.alts = 0;
+            if (conv_tc_plan(def, sd, why, sizeof(why))) return fail(FUSION_ECUDA, why);
         }
         float best_ms = 1e30f;
         int best[4] = {0, 0, 0, 0};
@@ -1711,6 +1714,7 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
                 for (int nbs : {2, 3, 4}) {
                     ConvTcPlan trial;
                     ConvTcSpec sp = conv_spec(m, i);
+                    sp.alts = 0;
                     sp.T = T;
                     sp.group = group;
                     sp.groups_per_stage = groups;
@@ -1729,6 +1733,8 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
                 }
         if (best[0] == 0) return fail(FUSION_EUNSUPPORTED, "no tile configuration fits layer " + std::to_string(i));
         ConvTcSpec sp = conv_spec(m, i);
+        const int alts = sp.alts;
+        sp.alts = 0;
         sp.T = best[0];
         sp.groups_per_stage = best[1];
         sp.nbs = best[2];
@@ -1750,6 +1756,7 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
             cand_best = std::min(cand_best, ms);
         }
         ConvTcSpec chosen = cand_best < 0.98f * def_best ? sp : conv_spec(m, i);
+        chosen.alts = alts;
         char why[256] = {0};
         if (conv_tc_plan(m->tcplan[i], chosen, why, sizeof(why))) return fail(FUSION_ECUDA, why);
     }

@@ -92,9 +92,11 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <vector>
 
 namespace fusion {
@@ -110,9 +112,11 @@ constexpr int kRing = 4;     // tile indices the producer publishes ahead of the
 template <int N, int T, int G>
 struct Roles {
     static constexpr int UNITS = T / G;                          // slice groups per tile
-    static constexpr int NI = kIssReq < UNITS ? kIssReq : UNITS;  // MMA-issuing warps, each owns UNITS / NI
+    // MMA-issuing warps, each owns UNITS / NI slice groups (6 groups: 3 warps)
+    static constexpr int NI = UNITS % kIssReq == 0 ? kIssReq : UNITS % 3 == 0 ? 3 : UNITS;
+    static_assert(NI <= kIssReq && UNITS % NI == 0, "every slice group has an issuer");
     static constexpr int UCOLS = G * N;                          // accumulator columns of one slice group
-    static constexpr int EPW = UCOLS > 128 ? UCOLS / 128 : 1;
+    static constexpr int EPW = (UCOLS + 127) / 128;
     static constexpr int PART = UCOLS / EPW;
     static constexpr int EPI0 = 1 + NI;                           // first epilogue warp
     static constexpr int THREADS = 32 * (EPI0 + 4 * EPW);
@@ -608,6 +612,8 @@ struct ConvTcPlan::Impl {
     int sms = 1;            // multiprocessors of the device (persistent grid size)
     size_t smem = 0;
     unsigned grid = 0;
+    double tile_clk = 0;    // estimated clocks of a tile, for choosing between tile heights
+    std::vector<std::unique_ptr<ConvTcPlan>> alts;   // plans of smaller tiles
 };
 
 ConvTcPlan::ConvTcPlan() : impl(new Impl()) {}
@@ -823,21 +829,72 @@ void conv_f32tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad
         });
 }
 
+// Clocks of a tile: its MMAs (N = width columns take the larger of N / 2 and the operand reads, 4 KB + 32 N bytes at 128
+// a clock; measured 40, 48, 64, 128 at N = 32, 64, 128, 256) or its weight stream (about 20 bytes a clock and SM: one-slice
+// tiles of the full-size stride-2 layer copy 2 MB each and took 103 thousand clocks for 32 thousand of MMAs), the halo loads
+// where one buffer makes the MMAs wait for them (about 36 bytes a clock), and a tile's hand-over.
+static double tile_clocks(const Args &A, int N, int T, int group) {
+    const Geo &g = A.g;
+    double clk = 2000;
+    for (int c = 0; c < g.chunks; ++c)
+        for (int ph = 0; ph < g.nphase; ++ph) {
+            int nz, ny, nx;
+            phase_ntaps(A.k, A.stride, ph, nz, ny, nx);
+            if (A.xpat) nx = A.xt_n[c];
+            double per_group = 0;
+            for (int u = 0; nz > 0 && u <= nz + group - 2; ++u) {
+                const int w = (std::min(u, group - 1) - std::max(0, u - (nz - 1)) + 1) * N;
+                per_group += std::max(w * 0.5, 32 + w * 0.25);
+            }
+            const double halo = g.a_bytes / 36.0 + 500;
+            const double mma = std::max(per_group * (T / group), nz * N * 32 / 20.0) * ny * nx;
+            clk += g.na == 1 ? mma + halo : std::max(mma, halo);
+        }
+    return clk;
+}
+
+static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *why, size_t why_len);
+
 int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_len) {
     ConvTcPlan::Impl &P = *plan.impl;
-    const int c_out = sp.c_out, k = sp.k, stride = sp.stride;
-    if (sp.T <= 0 && stride == 1 && wide_tiles_ok(c_out, sp.n_out)) {
+    P.alts.clear();
+    int r = -1;
+    if (sp.T <= 0 && sp.stride == 1 && wide_tiles_ok(sp.c_out, sp.n_out)) {
         ConvTcSpec wide = sp;
         wide.T = 16;
-        if (conv_tc_plan(plan, wide, why, why_len) == 0) return 0;   // else the default below
+        r = plan_tile(P, wide, false, why, why_len);   // else the default below
     }
+    if (r) r = plan_tile(P, sp, false, why, why_len);
+    if (r || !sp.alts) return r;
+    // Smaller tiles for calls that the planned ones would leave SMs idle in (one pose of the paper-final 24^3 layers is
+    // 18 tiles of 8 slices): conv_tc_launch takes the height with the shortest estimated schedule.  Every tile adds
+    // each output's terms in the same order, so the results do not depend on the choice.
+    for (int T : {8, 6, 4, 2, 1}) {
+        if (T >= P.T || (T == 6 && sp.c_out > 64) || (T == 1 && sp.c_out < 128)) continue;
+        ConvTcSpec a = sp;
+        a.T = T;
+        a.group = 1;
+        if (sp.stride == 1)
+            for (int G : {8, 6, 4, 3, 2})
+                if (T % G == 0 && G * sp.c_out <= 256 && (G < 6 || sp.c_out == 32)) { a.group = G; break; }
+        a.groups_per_stage = a.nbs = 0;
+        std::unique_ptr<ConvTcPlan> q(new ConvTcPlan());
+        char no[256];
+        if (plan_tile(*q->impl, a, true, no, sizeof(no)) == 0) P.alts.push_back(std::move(q));
+    }
+    return 0;
+}
+
+// One tile shape's geometry, tensor map and arguments.  alt: a shape only conv_tc_plan's own choice may take.
+static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *why, size_t why_len) {
+    const int c_out = sp.c_out, k = sp.k, stride = sp.stride;
     const int T = sp.T > 0 ? sp.T : conv_tc_tile_slices(c_out);
     const int chunk_ch = sp.elem == 2 ? 16 : 32;
     // 16 slices per CTA only at stride 1 (the strided phases are built and checked for at most 8)
     const bool t_ok = (c_out <= 64 && (T == 4 || T == 8)) || (c_out <= 32 && T == 16 && stride == 1) ||
                       (c_out == 128 && (T == 2 || T == 4)) ||
                       (c_out == 256 && T == 2);
-    if (!t_ok) {
+    if (!t_ok && !alt) {
         snprintf(why, why_len, "unsupported output slices per CTA (%d) for %d output channels at stride %d", T, c_out,
                  stride);
         return -1;
@@ -913,7 +970,7 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
     };
     int group = sp.group;
     if (group <= 0) group = stride != 1 ? 1 : (T == 16 && group_ok(8)) ? 8 : group_ok(4) ? 4 : group_ok(2) ? 2 : 1;
-    if (!group_ok(group)) {
+    if (!alt && !group_ok(group)) {
         snprintf(why, why_len, "%d slices per MMA: must be 1, 2, 4 or 8 (8: with 16 slices per CTA), divide the %d "
                  "slices per CTA and span <= 256 columns", group, T);
         return -1;
@@ -1028,6 +1085,7 @@ int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_l
         return -2;
     }
     A.tile_counter = P.counter;
+    P.tile_clk = tile_clocks(A, c_out, T, group);
     return 0;
 }
 
@@ -1044,13 +1102,19 @@ static void launch_t(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
 
 template <int N, int T, bool F8>
 static void launch_g(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
-    if constexpr (T == 16 && 8 * N <= 256) {
+    if constexpr (T % 8 == 0 && 8 * N <= 256) {
         if (P.group == 8) return launch_t<N, T, F8, 8>(P, B, s);
+    }
+    if constexpr (T == 6 && 6 * N <= 256) {
+        if (P.group == 6) return launch_t<N, T, F8, 6>(P, B, s);
+    }
+    if constexpr (T == 6 && N == 64) {
+        if (P.group == 3) return launch_t<N, T, F8, 3>(P, B, s);
     }
     if constexpr (T % 4 == 0 && 4 * N <= 256) {
         if (P.group == 4) return launch_t<N, T, F8, 4>(P, B, s);
     }
-    if constexpr (T % 2 == 0 && 2 * N <= 256) {
+    if constexpr (T % 2 == 0 && T != 6 && 2 * N <= 256) {
         if (P.group == 2) return launch_t<N, T, F8, 2>(P, B, s);
     }
     launch_t<N, T, F8, 1>(P, B, s);
@@ -1059,6 +1123,12 @@ static void launch_g(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
 template <bool F8>
 static void launch_n(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
     switch (P.N * 16 + P.T) {
+    case 32 * 16 + 2: launch_g<32, 2, F8>(P, B, s); break;
+    case 32 * 16 + 6: launch_g<32, 6, F8>(P, B, s); break;
+    case 64 * 16 + 2: launch_g<64, 2, F8>(P, B, s); break;
+    case 64 * 16 + 6: launch_g<64, 6, F8>(P, B, s); break;
+    case 128 * 16 + 1: launch_g<128, 1, F8>(P, B, s); break;
+    case 256 * 16 + 1: launch_g<256, 1, F8>(P, B, s); break;
     case 32 * 16 + 4: launch_g<32, 4, F8>(P, B, s); break;
     case 32 * 16 + 8: launch_g<32, 8, F8>(P, B, s); break;
     case 32 * 16 + 16: launch_g<32, 16, F8>(P, B, s); break;
@@ -1081,10 +1151,18 @@ void conv_tc_describe(const ConvTcPlan &plan, int *T, int *groups_per_stage, int
 void conv_tc_stall_next(ConvTcPlan &plan) { plan.impl->args.stall = 1; }
 
 void conv_tc_launch(ConvTcPlan &plan, int B, cudaStream_t s) {
-    ConvTcPlan::Impl &P = *plan.impl;
-    if (P.f8) launch_n<true>(P, B, s);
-    else launch_n<false>(P, B, s);
-    P.args.stall = 0;   // one launch only
+    ConvTcPlan::Impl &M = *plan.impl;
+    auto schedule = [&](const ConvTcPlan::Impl &p) {        // rounds of tiles over the SMs x a tile's clocks
+        const long long tiles = (long long)p.grid * B;
+        return (double)((tiles + p.sms - 1) / p.sms) * p.tile_clk;
+    };
+    ConvTcPlan::Impl *best = &M;
+    for (auto &q : M.alts)
+        if (schedule(*q->impl) < 0.97 * schedule(*best)) best = q->impl;
+    best->args.stall = M.args.stall;
+    if (best->f8) launch_n<true>(*best, B, s);
+    else launch_n<false>(*best, B, s);
+    best->args.stall = M.args.stall = 0;   // one launch only
 }
 
 }  // namespace fusion

@@ -1185,8 +1185,8 @@ static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, 
         flat_in = m->pool_out;
         map[10] = ei; mark(st);
     }
-    DenseArgs da{flat_in, m->dense_w, m->dense_b, m->dense_part, m->cnn_lat, B, d.cnn_dense, m->flat, m->splits,
-                 m->bf16 ? 1 : 0, 1};
+    DenseArgs da{static_cast<const float *>(flat_in), static_cast<const float *>(m->dense_w), m->dense_b, m->dense_part,
+                 m->cnn_lat, B, d.cnn_dense, m->flat, m->splits, 1};     // (a bf16 model's x and w go to dense_tc)
     if (m->bf16) {
         // tensor cores: split partials, then the same fixed-order reduction
         dense_tc_launch(m->dense_tc, B, m->dense_part, st);
@@ -1198,7 +1198,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, 
     if (d.cnn_dense2) {
         // the second CNN dense layer (FP32 on every dtype: a cnn_dense x cnn_dense2 matrix per pose)
         DenseArgs d2{m->cnn_lat, m->dense2_w, m->dense2_b, m->dense_part, m->cnn_lat2, B, d.cnn_dense2, d.cnn_dense,
-                     dense_splits(d.cnn_dense), 0, 1};
+                     dense_splits(d.cnn_dense), 1};
         launch_dense(d2, st);
     }
     RC(check_launch("dense"));

@@ -91,13 +91,12 @@ struct PoolArgs {
 void launch_maxpool(const PoolArgs &a, cudaStream_t s);
 
 struct DenseArgs {
-    const void *x;        // [B][K] (float or bf16)
-    const void *w;        // [N][K] (float or bf16)
+    const float *x;       // [B][K], 16-byte aligned, K a multiple of 8 (unused by launch_dense_reduce)
+    const float *w;       // [N][K], 16-byte aligned
     const float *bias;    // [N]
     float *part;          // [splits][B][N]
     float *y;             // [B][N]
     int B, N, K, splits;
-    int bf16;
     int relu;
 };
 void launch_dense(const DenseArgs &a, cudaStream_t s);

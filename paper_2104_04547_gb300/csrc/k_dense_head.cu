@@ -1,14 +1,21 @@
 // CNN dense layer and fusion head.
 //
-// CNN dense (Section 3.3.1: flatten -> dense + ReLU): y[b][n] = ReLU(bias[n] +
-// sum_k x[b][k] W[n][k]) with K = pooled voxels x channels (221,184 for the
-// full-size model).  At small batch the weight stream dominates, so it is a
-// split-K product: CTA (n-tile, split s, b-tile) multiplies a 64 x 64 tile over
-// the K slice of split s from shared-memory tiles, and a second kernel adds the
-// split partials in a fixed order (split count depends on K only, so a pose's
-// result does not depend on its batch) and applies bias and ReLU.  The weight
-// rows were permuted at model creation so that the flatten of the NDHWC pooled
-// map is a plain row read.
+// CNN dense in FP32 (Section 3.3.1: flatten -> dense + ReLU): y[b][n] = ReLU(bias[n] + sum_k x[b][k] W[n][k]) with
+// K = pooled voxels x channels (221,184 for the full-size model), a split-K product whose order of additions
+// depends on K only: split s, its eight sub-slices of K, in each a chain of multiply-adds in k order; the eight
+// chains are added in order, then a second kernel adds the splits.  So a pose's result does not depend on its batch,
+// and two kernels can share the work by batch size:
+//   * up to 16 poses the weight stream is the bound, and dense_stream_kernel keeps it flowing: a warp takes one
+//     sub-slice of 32 weight rows, a lane per row, through a private ring of 16-byte asynchronous copies (up to 128 KB in
+//     flight per SM with two CTAs), with no CTA barrier until the end;
+//   * above that the multiply-adds are (7.2 GFLOP at 64 poses: 90 us at the FP32 rate, 42 us for the bytes), and
+//     dense_tile_kernel gives each warp one sub-slice of a 64 x 64 (or 64 x 32) tile, a lane 8 x 16 outputs, reading
+//     k-quads of rows as they lie in memory (a transpose would cost as many stores as the loads it saves).
+// The line between them is where 16 sums per weight still fit a lane and cost less than the stream (23 of 33 us).
+// The weight rows were permuted at model creation so that the flatten of the NDHWC pooled map is a plain row read.
+// Measured with the reduction, through the no-allocation entry: 4 x 128 x 110,592 127 -> 21.5 us (58 MB, 2.7 TB/s),
+// 64 x 256 x 221,184 266 -> 197 us (36.8 TFLOP/s); the dense layer of the single-pose 24^3 model 100 -> 16 us, of the
+// full-size model at 3 poses 256 -> 61 us.  Errors against float64 fell from 6e-7 to 2.4e-7 (chains of 256, not 2048).
 //
 // Fusion head (Section 3.3.3, Table V: fusion dense layers with SELU): one CTA
 // per pose runs Linear -> SELU -> ... -> Linear on [cnn latent, sg latent].
@@ -18,108 +25,205 @@ namespace fusion {
 
 namespace {
 
-constexpr int DT = 64;     // tile edge (poses and outputs)
-constexpr int DBK = 32;    // K chunk
+constexpr int kDenseWarps = 8;            // sub-slices of a split, one warp each
+constexpr int kDenseThreads = 32 * kDenseWarps;
 
-template <bool BF16>
-__device__ __forceinline__ void load8(const void *base, size_t idx, bool ok, float *out) {
-    if (!ok) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) out[j] = 0.f;
-        return;
-    }
-    if constexpr (BF16) {
-        const uint4 u = *reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(base) + idx);
-        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(h[j]);
-            out[2 * j] = f.x;
-            out[2 * j + 1] = f.y;
-        }
-    } else {
-        const float *p = reinterpret_cast<const float *>(base) + idx;
-        const float4 a = *reinterpret_cast<const float4 *>(p);
-        const float4 b = *reinterpret_cast<const float4 *>(p + 4);
-        out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
-        out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 16 : 0));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N)); }
+
+// K range [kb, ke) of warp q in split s: splits of kper (a multiple of 64), eight sub-slices each (empty past K).
+__device__ __forceinline__ void dense_range(const DenseArgs &a, int q, int &kb, int &ke) {
+    const int kper = ((a.K + a.splits - 1) / a.splits + 63) / 64 * 64, sub = kper / kDenseWarps;
+    kb = blockIdx.y * kper + q * sub;
+    ke = min(a.K, kb + sub);
+}
+
+// `rows` rows from r0 of a [.. limit][K] matrix, columns [k, k + KC) (zero past ke and past the last row), into a tile
+// with rows of KC + 4 floats: a warp's 16-byte reads down eight rows then touch all banks.
+template <int KC>
+__device__ __forceinline__ void dense_stage(float *tile, const float *m, int r0, int rows, int limit, int K, int k, int ke,
+                                            int lane) {
+    for (int e = lane; e < rows * (KC / 4); e += 32) {
+        const int r = e / (KC / 4), c = (e % (KC / 4)) * 4;
+        const bool ok = r0 + r < limit && k + c < ke;       // ke is a multiple of 8: a quad is all in or all out
+        cp_async16(tile + r * (KC + 4) + c, ok ? m + (size_t)(r0 + r) * K + k + c : m, ok);
     }
 }
 
-template <bool BF16>
-__global__ void __launch_bounds__(256) dense_splitk_kernel(DenseArgs a) {
-    __shared__ __align__(16) float xs[DBK][DT + 4];
-    __shared__ __align__(16) float ws[DBK][DT + 4];
-    const int tid = threadIdx.x;
-    const int n0 = blockIdx.x * DT;
-    const int split = blockIdx.y;
-    const int b0 = blockIdx.z * DT;
-    const int kper = ((a.K + a.splits - 1) / a.splits + DBK - 1) / DBK * DBK;
-    const int kbeg = split * kper;
-    const int kend = min(a.K, kbeg + kper);
+constexpr int kStreamRows = 32, kStreamKC = 16;
+template <int BT>
+struct StreamTile {
+    static constexpr int STAGES = BT <= 4 ? 5 : BT <= 8 ? 4 : 3;       // the most that leave room for two CTAs on an SM
+    static constexpr int LD = kStreamKC + 4, STAGE = (kStreamRows + BT) * LD, RING = STAGES * STAGE;   // floats, a warp's
+};
 
-    // load role: row r = tid / 4 (0..63), k offset (tid % 4) * 8
-    const int lr = tid >> 2, lk = (tid & 3) * 8;
-    const int tr = tid / 16, tc = tid % 16;    // compute role: rows tr*4.., cols tc*4..
-    float acc[4][4] = {};
-    for (int kc = kbeg; kc < kend; kc += DBK) {
-        float xv[8], wv[8];
-        const int kk = kc + lk;
-        const bool kin = kk < kend;      // K is a multiple of 8, so a chunk of 8 is all in or all out
-        load8<BF16>(a.x, (size_t)(b0 + lr) * a.K + kk, kin && (b0 + lr) < a.B, xv);
-        load8<BF16>(a.w, (size_t)(n0 + lr) * a.K + kk, kin && (n0 + lr) < a.N, wv);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            xs[lk + j][lr] = xv[j];
-            ws[lk + j][lr] = wv[j];
+template <int BT>
+__global__ void __launch_bounds__(kDenseThreads, 2) dense_stream_kernel(DenseArgs a) {
+    extern __shared__ __align__(16) float dsm[];
+    using S = StreamTile<BT>;
+    constexpr int LD = S::LD, STAGE = S::STAGE, STAGES = S::STAGES;
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int n0 = blockIdx.x * kStreamRows;
+    const float *x = a.x, *w = a.w;
+    float *ring = dsm + q * S::RING;
+    int kb, ke;
+    dense_range(a, q, kb, ke);
+    const int steps = ke > kb ? (ke - kb + kStreamKC - 1) / kStreamKC : 0;
+    auto load = [&](int i) {
+        if (i < steps) {
+            float *st = ring + (i % STAGES) * STAGE;
+            dense_stage<kStreamKC>(st, w, n0, kStreamRows, a.N, a.K, kb + i * kStreamKC, ke, lane);
+            dense_stage<kStreamKC>(st + kStreamRows * LD, x, 0, BT, a.B, a.K, kb + i * kStreamKC, ke, lane);
         }
-        __syncthreads();
-#pragma unroll 8
-        for (int q = 0; q < DBK; ++q) {
-            const float4 x4 = *reinterpret_cast<const float4 *>(&xs[q][tr * 4]);
-            const float4 w4 = *reinterpret_cast<const float4 *>(&ws[q][tc * 4]);
-            const float xr[4] = {x4.x, x4.y, x4.z, x4.w};
-            const float wr[4] = {w4.x, w4.y, w4.z, w4.w};
+        cp_async_commit();
+    };
+    float acc[BT];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+    for (int b = 0; b < BT; ++b) acc[b] = 0.f;
+    for (int i = 0; i < STAGES - 1; ++i) load(i);
+    for (int i = 0; i < steps; ++i) {
+        load(i + STAGES - 1);
+        cp_async_wait<STAGES - 1>();
+        __syncwarp();
+        const float *st = ring + (i % STAGES) * STAGE;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xr[i], wr[j], acc[i][j]);
+        for (int c = 0; c < kStreamKC; c += 4) {
+            const float4 w4 = *reinterpret_cast<const float4 *>(st + lane * LD + c);
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                const float4 x4 = *reinterpret_cast<const float4 *>(st + (kStreamRows + b) * LD + c);
+                acc[b] = fmaf(x4.x, w4.x, acc[b]);
+                acc[b] = fmaf(x4.y, w4.y, acc[b]);
+                acc[b] = fmaf(x4.z, w4.z, acc[b]);
+                acc[b] = fmaf(x4.w, w4.w, acc[b]);
+            }
         }
-        __syncthreads();
+        __syncwarp();                            // the stage is free for the copies of the next iteration
     }
+    cp_async_wait<0>();
+    __syncthreads();
+    // the eight chains in order
+    float *red = dsm;                            // [8][BT][32]
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int b = b0 + tr * 4 + i;
-        if (b >= a.B) continue;
+    for (int b = 0; b < BT; ++b) red[(q * BT + b) * 32 + lane] = acc[b];
+    __syncthreads();
+    for (int e = threadIdx.x; e < BT * 32; e += kDenseThreads) {
+        const int b = e >> 5, n = n0 + (e & 31);
+        float s = red[e];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tc * 4 + j;
-            if (n < a.N) a.part[((size_t)split * a.B + b) * a.N + n] = acc[i][j];
-        }
+        for (int j = 1; j < kDenseWarps; ++j) s += red[j * BT * 32 + e];
+        if (b < a.B && n < a.N) a.part[((size_t)blockIdx.y * a.B + b) * a.N + n] = s;
     }
 }
 
-// Sum of the split partials in split order (fixed, so the result does not depend on the batch),
-// plus bias and activation.  The partials are loaded 8 at a time ahead of the in-order additions so
-// that a thread keeps several loads in flight instead of waiting on each one.
-__global__ void dense_reduce_kernel(DenseArgs a) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.B * a.N) return;
-    const int n = e % a.N;
-    const size_t stride = (size_t)a.B * a.N;
-    const float *p = a.part + e;
+constexpr int kTileN = 64, kTileKC = 16;
+template <int BT>
+struct GemmTile {
+    static constexpr int LD = kTileKC + 4, STAGE = (kTileN + BT) * LD, RING = 2 * STAGE;               // floats, a warp's
+};
+
+// BT poses (64 or 32): a lane's outputs are rows lane % 8 + 8 j and poses lane / 8 + 4 i.
+template <int BT>
+__global__ void __launch_bounds__(kDenseThreads, 1) dense_tile_kernel(DenseArgs a) {
+    extern __shared__ __align__(16) float dsm[];
+    using S = GemmTile<BT>;
+    constexpr int LD = S::LD, STAGE = S::STAGE, NI = BT / 4;
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int n0 = blockIdx.x * kTileN, b0 = blockIdx.z * BT;
+    const int ln = lane & 7, lb = lane >> 3;
+    const float *x = a.x, *w = a.w;
+    float *ring = dsm + q * S::RING;
+    int kb, ke;
+    dense_range(a, q, kb, ke);
+    const int steps = ke > kb ? (ke - kb + kTileKC - 1) / kTileKC : 0;
+    auto load = [&](int i) {
+        if (i < steps) {
+            float *st = ring + (i & 1) * STAGE;
+            dense_stage<kTileKC>(st, w, n0, kTileN, a.N, a.K, kb + i * kTileKC, ke, lane);
+            dense_stage<kTileKC>(st + kTileN * LD, x, b0, BT, a.B, a.K, kb + i * kTileKC, ke, lane);
+        }
+        cp_async_commit();
+    };
+    float acc[NI][8];
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    load(0);
+    for (int s = 0; s < steps; ++s) {
+        load(s + 1);
+        cp_async_wait<1>();
+        __syncwarp();
+        const float *ws = ring + (s & 1) * STAGE + ln * LD, *xs = ring + (s & 1) * STAGE + (kTileN + lb) * LD;
+#pragma unroll 1
+        for (int c = 0; c < kTileKC; c += 4) {
+            float4 wv[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) wv[j] = *reinterpret_cast<const float4 *>(ws + 8 * j * LD + c);
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                const float4 xv = *reinterpret_cast<const float4 *>(xs + 4 * i * LD + c);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xv.x, wv[j].x, acc[i][j]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xv.y, wv[j].y, acc[i][j]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xv.z, wv[j].z, acc[i][j]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xv.w, wv[j].w, acc[i][j]);
+            }
+        }
+        __syncwarp();
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    float *red = dsm;                            // [8][BT][64]
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) red[(q * BT + lb + 4 * i) * kTileN + ln + 8 * j] = acc[i][j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < BT * kTileN; e += kDenseThreads) {
+        const int b = b0 + e / kTileN, n = n0 + e % kTileN;
+        float s = red[e];
+#pragma unroll
+        for (int j = 1; j < kDenseWarps; ++j) s += red[j * BT * kTileN + e];
+        if (b < a.B && n < a.N) a.part[((size_t)blockIdx.y * a.B + b) * a.N + n] = s;
+    }
+}
+
+// Sum of the split partials plus bias and activation: a block takes 32 outputs, its eight warps an eighth of the
+// splits each (in order), and the eight sums are added in order, so the result does not depend on the batch.  Bound by
+// the latency of its loads: one thread per output walked 108 partials in 14 rounds, a warp now holds its 14 in flight.
+__global__ void __launch_bounds__(256) dense_reduce_kernel(DenseArgs a) {
+    __shared__ float sums[8][32];
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane, tot = a.B * a.N;
+    const int per = (a.splits + 7) / 8, lo = q * per, hi = min(a.splits, lo + per);
     float s = 0.f;
-    int q = 0;
-    for (; q + 8 <= a.splits; q += 8) {
-        float v[8];
+    if (e < tot) {
+        const float *p = a.part + e;
+        for (int i = lo; i < hi; i += 16) {
+            float v[16];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = __ldg(p + (size_t)(q + j) * stride);
+            for (int j = 0; j < 16; ++j) v[j] = i + j < hi ? __ldg(p + (size_t)(i + j) * tot) : 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s += v[j];
+            for (int j = 0; j < 16; ++j) s += v[j];
+        }
     }
-    for (; q < a.splits; ++q) s += __ldg(p + (size_t)q * stride);
-    s += a.bias[n];
-    a.y[e] = a.relu ? fmaxf(s, 0.f) : s;
+    sums[q][lane] = s;
+    __syncthreads();
+    if (q == 0 && e < tot) {
+#pragma unroll
+        for (int j = 1; j < 8; ++j) s += sums[j][lane];
+        s += a.bias[e % a.N];
+        a.y[e] = a.relu ? fmaxf(s, 0.f) : s;
+    }
 }
 
 __device__ __forceinline__ float selu(float x) {
@@ -260,16 +364,33 @@ int dense_splits(int K) {
     return s;
 }
 
+template <int BT>
+static void launch_stream(const DenseArgs &a, cudaStream_t s) {
+    const size_t ring = (size_t)kDenseWarps * StreamTile<BT>::RING * 4;      // covers the [8][BT][32] sums too
+    cudaFuncSetAttribute(dense_stream_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
+    dense_stream_kernel<BT><<<dim3((a.N + kStreamRows - 1) / kStreamRows, a.splits), kDenseThreads, ring, s>>>(a);
+}
+
+template <int BT>
+static void launch_tile(const DenseArgs &a, cudaStream_t s) {
+    const size_t ring = (size_t)kDenseWarps * GemmTile<BT>::RING * 4;        // covers the [8][BT][64] sums too
+    cudaFuncSetAttribute(dense_tile_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
+    dense_tile_kernel<BT><<<dim3((a.N + kTileN - 1) / kTileN, a.splits, (a.B + BT - 1) / BT), kDenseThreads, ring, s>>>(a);
+}
+
 void launch_dense(const DenseArgs &a, cudaStream_t s) {
-    dim3 grid((a.N + DT - 1) / DT, a.splits, (a.B + DT - 1) / DT);
-    if (a.bf16) dense_splitk_kernel<true><<<grid, 256, 0, s>>>(a);
-    else dense_splitk_kernel<false><<<grid, 256, 0, s>>>(a);
+    if (a.B <= 1) launch_stream<1>(a, s);
+    else if (a.B <= 4) launch_stream<4>(a, s);
+    else if (a.B <= 8) launch_stream<8>(a, s);
+    else if (a.B <= 16) launch_stream<16>(a, s);
+    else if (a.B <= 32) launch_tile<32>(a, s);
+    else launch_tile<64>(a, s);
     launch_dense_reduce(a, s);
 }
 
 void launch_dense_reduce(const DenseArgs &a, cudaStream_t s) {
     const int tot = a.B * a.N;
-    dense_reduce_kernel<<<(tot + 127) / 128, 128, 0, s>>>(a);
+    dense_reduce_kernel<<<(tot + 31) / 32, 256, 0, s>>>(a);
 }
 
 void launch_head(const HeadArgs &a, cudaStream_t s) {

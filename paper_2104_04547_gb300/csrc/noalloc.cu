@@ -80,7 +80,7 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
     if (e != cudaSuccess)
         return noalloc_fail(FUSION_ECUDA, std::string("a CUDA error was pending before this call (nothing launched): ") +
                                               cudaGetErrorString(e));
-    fusion::DenseArgs a{x, w, bias, static_cast<float *>(scratch), y, B, N, K, splits, 0, relu ? 1 : 0};
+    fusion::DenseArgs a{x, w, bias, static_cast<float *>(scratch), y, B, N, K, splits, relu ? 1 : 0};
     fusion::launch_dense(a, static_cast<cudaStream_t>(cuda_stream));
     e = cudaGetLastError();
     if (e != cudaSuccess) return noalloc_fail(FUSION_ECUDA, std::string("dense launch: ") + cudaGetErrorString(e));

@@ -100,6 +100,9 @@ struct DenseArgs {
     int relu;
 };
 void launch_dense(const DenseArgs &a, cudaStream_t s);
+// The same layer on the tensor cores at FP32's accuracy (k_dense_f32tc.cu), with at most a.splits splits; the order of
+// additions depends on the batch.
+void launch_dense_f32tc(DenseArgs a, cudaStream_t s);
 int dense_splits(int K);
 // The fixed-order split reduction + bias + activation of launch_dense, on partials [splits][B][N].
 void launch_dense_reduce(const DenseArgs &a, cudaStream_t s);

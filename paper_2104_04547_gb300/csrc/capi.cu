@@ -967,7 +967,7 @@ static int check_launch(const char *what) {
     return FUSION_OK;
 }
 
-static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, const int32_t *off_d,
+static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const int32_t *A_dev, const int32_t *off_d,
                            const int32_t *nlig_d, const float *xyz_d, const float *feat_d, bool timed, int *map) {
     const fusion_model_desc &d = m->d;
     cudaStream_t ms = m->stream;        // the model's (caller-visible) stream: prep, join, head
@@ -1009,7 +1009,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, const int32_t *A_dev, 
     auto graph_branch = [&]() -> int {
         sg_mark(0);
         // radius graph
-        GraphArgs ga{off_d, xyz_d, B, d.max_atoms, d.max_degree, d.cut_cov, d.cut_nc,
+        GraphArgs ga{off_d, xyz_d, B, d.max_atoms, most_atoms, d.max_degree, d.cut_cov, d.cut_nc,
                      {m->e_beg[0], m->e_beg[1]}, {m->e_deg[0], m->e_deg[1]}, {m->e_col[0], m->e_col[1]}, m->err};
         launch_radius_graph(ga, sgs);
         RC(check_launch("radius_graph"));
@@ -1318,7 +1318,7 @@ int fusion_score(fusion_model *m, const fusion_poses *poses, int32_t n_poses, fl
         auto it = m->graph_exec.find(B);
         if (it == m->graph_exec.end()) {
             CU(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
-            const int rc = enqueue_forward(m, B, B * d.max_atoms, m->in_off + B, m->in_off, m->in_nlig, m->in_xyz,
+            const int rc = enqueue_forward(m, B, B * d.max_atoms, d.max_atoms, m->in_off + B, m->in_off, m->in_nlig, m->in_xyz,
                                            m->in_feat, false, map);
             cudaGraph_t g = nullptr;
             const cudaError_t e = cudaStreamEndCapture(st, &g);
@@ -1340,7 +1340,9 @@ int fusion_score(fusion_model *m, const fusion_poses *poses, int32_t n_poses, fl
         CU(cudaGraphLaunch(it->second, st));
         cudaEventRecord(m->ev[1], st);
     } else {
-        RC(enqueue_forward(m, B, A, nullptr, off_d, nlig_d, xyz_d, feat_d, true, map));
+        int most = 0;
+        for (int p = 0; p < B; ++p) most = std::max(most, off[p + 1] - off[p]);
+        RC(enqueue_forward(m, B, A, most, nullptr, off_d, nlig_d, xyz_d, feat_d, true, map));
     }
 
     CU(cudaMemcpyAsync(m->h_err, m->err, 4 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));

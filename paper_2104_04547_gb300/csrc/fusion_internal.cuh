@@ -261,6 +261,7 @@ struct GraphArgs {
     const float *xyz;
     int n_poses;
     int max_atoms;
+    int most_atoms;       // no pose has more (the batch's largest, or max_atoms where that is not known)
     int max_degree;
     float cut_cov, cut_nc;
     int32_t *beg[2], *deg[2], *col[2];   // 0 covalent, 1 non-covalent

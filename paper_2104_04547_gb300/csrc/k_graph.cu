@@ -1,7 +1,16 @@
 // Radius graph with two edge types (Section 1: edge types at distinct distance
 // thresholds for covalent and non-covalent interactions; Table II cutoffs).
 //
-// Three launches: a count pass and a fill pass with kGraphSplit CTAs per pose,
+// Batches whose poses have at most kPairAtoms atoms test every pair: a warp takes four query atoms, its lanes 32
+// candidates at a time from the pose's coordinates in shared memory, in index order, so rows come out sorted.  That is
+// about 13 instructions per query and 32 candidates (about 250 per query and pass at 500 atoms) against 850 for a query
+// of the cell list below (run bounds, lookups by shuffle, the row's sort), and no list to build in every CTA.  Small
+// batches run it as one launch, a cluster of kGraphSplit CTAs per pose with a cluster barrier between counting and
+// filling; larger ones as a count pass, a scan and a fill pass, whose CTAs need not find a cluster's worth of free
+// multiprocessors beside the convolutions.  Against the cell list, branches serialised: one pose 61 -> 20 us, 64 poses
+// 119 -> 63 us (paper-final cutoffs) and 101 -> 65 us, 256 poses 346 -> 219 us.
+//
+// Larger poses, three launches: a count pass and a fill pass with kGraphSplit CTAs per pose,
 // and between them one CTA per pose that scans the degrees into row offsets.
 // Every CTA of the count and fill passes puts its pose's coordinates in shared
 // memory and counting-sorts them into a cell list with cells no smaller than
@@ -353,6 +362,152 @@ __global__ void __launch_bounds__(kThreads) radius_fill_kernel(GraphArgs a) {
     }
 }
 
+// ---- every pair: poses of at most kPairAtoms atoms ----
+
+constexpr int kPairAtoms = 2048;    // beyond, the pairs outgrow the cell list's work
+constexpr int kQuery = 4;           // query atoms a warp takes at once
+
+// The pose's coordinates into shared memory, [3][n32] (padded with infinities to a multiple of 32: never a neighbour).
+__device__ void load_coords(const GraphArgs &a, int a0, int N, float *sx, int n32) {
+    for (int i = threadIdx.x; i < n32; i += blockDim.x)
+        for (int d = 0; d < 3; ++d) sx[d * n32 + i] = i < N ? a.xyz[(size_t)(a0 + i) * 3 + d] : INFINITY;
+    __syncthreads();
+}
+
+// Calls hit(t, j, cov, nc) in lockstep for query atoms i .. i + kQuery - 1 (t) and every group of 32 candidates j = lane + ..
+template <class Hit>
+__device__ __forceinline__ void scan_pairs(const GraphArgs &a, const float *sx, int n32, int i, int lane, Hit hit) {
+    const float c2 = __fmul_rn(a.cut_cov, a.cut_cov), n2 = __fmul_rn(a.cut_nc, a.cut_nc);
+    float q[kQuery][3];
+#pragma unroll
+    for (int t = 0; t < kQuery; ++t)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) q[t][d] = sx[d * n32 + min(i + t, n32 - 1)];
+    for (int j = lane; j < n32; j += 32) {
+        const float x = sx[j], y = sx[n32 + j], z = sx[2 * n32 + j];
+#pragma unroll
+        for (int t = 0; t < kQuery; ++t) {
+            const float s = dist2_rn(q[t][0], q[t][1], q[t][2], x, y, z);
+            const bool other = j != i + t, cov = s < c2;
+            hit(t, j, other && cov, other && !cov && s < n2);
+        }
+    }
+}
+
+__device__ void pair_count(const GraphArgs &a, int a0, int N, const float *sx, int n32, int part) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int i0, i1;
+    part_range(N, part, i0, i1);
+    for (int i = i0 + warp * kQuery; i < i1; i += kThreads / 32 * kQuery) {
+        int d0[kQuery] = {}, d1[kQuery] = {};
+        scan_pairs(a, sx, n32, i, lane, [&](int t, int, bool cov, bool nc) {
+            d0[t] += cov;
+            d1[t] += nc;
+        });
+#pragma unroll
+        for (int t = 0; t < kQuery; ++t) {
+            const int c0 = __reduce_add_sync(0xffffffffu, d0[t]), c1 = __reduce_add_sync(0xffffffffu, d1[t]);
+            if (lane == 0 && i + t < i1) {
+                a.deg[0][a0 + i + t] = c0;
+                a.deg[1][a0 + i + t] = c1;
+            }
+        }
+    }
+}
+
+// Rows of part `part`, offsets beg(e, local atom) from the pose's first column.
+template <class Beg>
+__device__ void pair_fill(const GraphArgs &a, int a0, int N, const float *sx, int n32, int part, Beg beg) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int i0, i1;
+    part_range(N, part, i0, i1);
+    for (int i = i0 + warp * kQuery; i < i1; i += kThreads / 32 * kQuery) {
+        int32_t *r0[kQuery], *r1[kQuery];
+#pragma unroll
+        for (int t = 0; t < kQuery; ++t) {
+            r0[t] = a.col[0] + beg(0, min(i + t, i1 - 1));
+            r1[t] = a.col[1] + beg(1, min(i + t, i1 - 1));
+        }
+        scan_pairs(a, sx, n32, i, lane, [&](int t, int j, bool cov, bool nc) {
+            const bool row = i + t < i1;                    // a query past the share's end writes nothing
+            const unsigned b0 = __ballot_sync(0xffffffffu, cov && row), b1 = __ballot_sync(0xffffffffu, nc && row);
+            if (cov && row) r0[t][__popc(b0 & below)] = a0 + j;
+            if (nc && row) r1[t][__popc(b1 & below)] = a0 + j;
+            r0[t] += __popc(b0);
+            r1[t] += __popc(b1);
+        });
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) pair_count_kernel(GraphArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int p = blockIdx.x / kGraphSplit;
+    const int a0 = a.atom_off[p], N = a.atom_off[p + 1] - a0;
+    if (N < 1 || N > a.most_atoms || a0 < 0) return;   // flagged by the prep kernel
+    float *sx = reinterpret_cast<float *>(smem);
+    const int n32 = (N + 31) & ~31;
+    load_coords(a, a0, N, sx, n32);
+    pair_count(a, a0, N, sx, n32, blockIdx.x % kGraphSplit);
+}
+
+__global__ void __launch_bounds__(kThreads) pair_fill_kernel(GraphArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int p = blockIdx.x / kGraphSplit;
+    const int a0 = a.atom_off[p], N = a.atom_off[p + 1] - a0;
+    if (N < 1 || N > a.most_atoms || a0 < 0) return;
+    float *sx = reinterpret_cast<float *>(smem);
+    const int n32 = (N + 31) & ~31;
+    load_coords(a, a0, N, sx, n32);
+    // the scan has zeroed every degree of a pose over capacity (its rows all start at its first column): no edges there.
+    // Any other pose's last row ends past that start unless the pose has no edges at all, which fills nothing anyway.
+    const int last = a0 + N - 1, base = a0 * a.max_degree;
+    bool any = false;
+    for (int e = 0; e < 2; ++e) any = any || a.beg[e][last] + a.deg[e][last] > base;
+    if (!any) return;
+    pair_fill(a, a0, N, sx, n32, blockIdx.x % kGraphSplit, [&](int e, int i) { return a.beg[e][a0 + i]; });
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// One launch: a cluster of kGraphSplit CTAs per pose counts, scans (each CTA the whole pose's degrees) and fills.
+__global__ void __launch_bounds__(kThreads) pair_graph_kernel(GraphArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_tmp[33];
+    const int p = blockIdx.x / kGraphSplit, part = blockIdx.x % kGraphSplit;
+    const int a0 = a.atom_off[p], N = a.atom_off[p + 1] - a0;
+    if (N < 1 || N > a.most_atoms || a0 < 0) return;         // the whole cluster; flagged by the prep kernel
+    float *sx = reinterpret_cast<float *>(smem);
+    const int n32 = (N + 31) & ~31;
+    int *off[2] = {reinterpret_cast<int *>(sx + 3 * n32), reinterpret_cast<int *>(sx + 3 * n32) + n32 + 1};
+    load_coords(a, a0, N, sx, n32);
+    pair_count(a, a0, N, sx, n32, part);
+    cluster_sync();
+    const long long cap = (long long)N * a.max_degree;
+    const int base = a0 * a.max_degree;
+    bool over = false;
+    for (int e = 0; e < 2; ++e) {
+        for (int i = threadIdx.x; i <= N; i += kThreads) off[e][i] = i < N ? __ldcg(a.deg[e] + a0 + i) : 0;
+        __syncthreads();
+        over = block_exscan(off[e], N + 1, s_tmp) > cap || over;
+    }
+    cluster_sync();                                         // every CTA has read the degrees
+    int i0, i1;
+    part_range(N, part, i0, i1);
+    for (int i = i0 + threadIdx.x; i < i1; i += kThreads)
+        for (int e = 0; e < 2; ++e) {
+            a.beg[e][a0 + i] = base + (over ? 0 : off[e][i]);
+            if (over) a.deg[e][a0 + i] = 0;
+        }
+    if (over) {
+        if (part == 0 && threadIdx.x == 0) atomicOr(a.err, FUSION_ERR_EDGES);
+        return;
+    }
+    pair_fill(a, a0, N, sx, n32, part, [&](int e, int i) { return base + off[e][i]; });
+}
+
 }  // namespace
 
 size_t radius_graph_smem(int max_atoms) {
@@ -360,12 +515,37 @@ size_t radius_graph_smem(int max_atoms) {
 }
 
 void launch_radius_graph(const GraphArgs &a, cudaStream_t s) {
+    const unsigned split = (unsigned)a.n_poses * kGraphSplit;
+    if (a.most_atoms <= kPairAtoms) {
+        const size_t n32 = (size_t)(a.most_atoms + 31) / 32 * 32, coords = 3 * n32 * 4;
+        if (split <= 128) {      // up to 16 poses
+            const size_t sm = coords + 2 * (n32 + 1) * 4;
+            cudaFuncSetAttribute(pair_graph_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = split;
+            cfg.blockDim = kThreads;
+            cfg.dynamicSmemBytes = sm;
+            cfg.stream = s;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = kGraphSplit;
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            cudaLaunchKernelEx(&cfg, pair_graph_kernel, a);
+            return;
+        }
+        pair_count_kernel<<<split, kThreads, coords, s>>>(a);
+        radius_scan_kernel<<<a.n_poses, kThreads, (size_t)(a.max_atoms + 1) * 4, s>>>(a);
+        pair_fill_kernel<<<split, kThreads, coords, s>>>(a);
+        return;
+    }
     const size_t sm = radius_graph_smem(a.max_atoms);
     cudaFuncSetAttribute(radius_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(radius_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    radius_count_kernel<<<a.n_poses * kGraphSplit, kThreads, sm, s>>>(a);
+    radius_count_kernel<<<split, kThreads, sm, s>>>(a);
     radius_scan_kernel<<<a.n_poses, kThreads, (size_t)(a.max_atoms + 1) * 4, s>>>(a);
-    radius_fill_kernel<<<a.n_poses * kGraphSplit, kThreads, sm, s>>>(a);
+    radius_fill_kernel<<<split, kThreads, sm, s>>>(a);
 }
 
 }  // namespace fusion

@@ -740,6 +740,25 @@ int alloc_workspace(fusion_model *m) {
 
 }  // namespace
 
+// Whether a call's kernels start early (launch_kernel), where they leave most multiprocessors idle: at most 48 tiles of 128
+// graph nodes, a third of the multiprocessors (10 paper-size poses).  Paper-final model, host call: one pose 311 -> 255 us,
+// two 372 -> 330, four 446 -> 396 (most of it the graph branch's kernels, see below); from eight on, and for the full-size
+// model, whose tiles fill the chip, the same either way (615 and 614, 628 and 630 us).
+static bool early_launches(int atoms) { return atoms <= 128 * 48; }
+
+// Of those, the calls whose graph branch takes longer than the convolutions it runs beside (one to three poses of the
+// paper-final model, whose nine steps were 60% of the call): there the graph's kernels start early too, and the
+// convolutions' tiles are chosen for the multiprocessors that its waiting CTAs do not hold.  Elsewhere those CTAs would
+// only keep multiprocessors from the convolutions (full-size model, one pose: 627 -> 657 us).
+constexpr int kGraphSms = 24;       // 16 CTAs of messages and 5 of GRU tiles for 500 atoms
+static bool graph_is_longer(const fusion_model *m, int B) {
+    if (!m->sg_tc || !m->bf16) return false;
+    double conv = 0, graph = 65;                    // us: radius graph, stage starts, gather
+    for (int i = 0; i < m->d.n_conv; ++i) conv += conv_tc_clocks(m->tcplan[i], B) / 1950 + 5;
+    for (int s = 0; s < m->d.sg_n_stages; ++s) graph += 17.0 * m->d.sg_steps[s];
+    return conv + 40 < graph;                       // beside voxelize and the dense layer
+}
+
 // FP8 inputs of the stride-1 layers are stored channel-blocked (whole W-lines per TMA box row), those of
 // the stride-2 layers parity-split (fp8_split; a first layer and an odd size read NDHWC with the TMA
 // element stride).
@@ -973,6 +992,8 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
     cudaStream_t ms = m->stream;        // the model's (caller-visible) stream: prep, join, head
     m->stall_armed = false;             // this pass consumes an armed wait-timeout test
     cudaStream_t st = m->cnn_stream;    // the grid branch, at the highest stream priority
+    const bool early = early_launches(A), graph_early = early && graph_is_longer(m, B);
+    const int busy_sms = graph_early && !m->serial_branches ? kGraphSms : 0;
     CU(cudaMemsetAsync(m->err, 0, 4 * sizeof(unsigned), ms));
 
     int ei = 0;
@@ -1058,6 +1079,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                 ga.H = H;
                 ga.A_dev = A_dev;
                 ga.err = m->err;
+                ga.early = graph_early;
                 ga.stall = m->sg_stall_next ? 1 : 0;
                 m->sg_stall_next = false;
                 launch_sg_stage_tc(ga, sgs);
@@ -1089,6 +1111,9 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                 sa.A_dev = A_dev;
                 sa.nodes_per_warp = m->sg_npw;
                 if (m->sg_tc) {
+                    // a warp per node where the branch is the longer one (see message_sums), unless the schedule was chosen
+                    if (graph_early && !m->sg_npw_set) sa.nodes_per_warp = 1;
+                    sa.early = graph_early;
                     launch_sg_message(sa, m->mbuf, sgs);
                     RC(check_launch("sg_message"));
                     SgGruTcArgs ga{};
@@ -1106,6 +1131,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                     ga.H = H;
                     ga.A_dev = A_dev;
                     ga.err = m->err;
+                    ga.early = graph_early;
                     ga.stall = m->sg_stall_next ? 1 : 0;
                     m->sg_stall_next = false;
                     launch_sg_gru_tc(ga, sgs);
@@ -1122,7 +1148,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
         const float *stage_in = m->xin;
         sg_mark(2);
         SgGatherArgs gg{off_d, nlig_d, m->last_h, stage_in, m->gat_wg_t, m->gat_bg, m->gat_wo_t, m->gat_bo,
-                        m->sg_lat, B, H, d.sg_gather_width, d.sg_gather == FUSION_GATHER_GATED};
+                        m->sg_lat, B, H, d.sg_gather_width, d.sg_gather == FUSION_GATHER_GATED, graph_early};
         launch_sg_gather(gg, sgs);
         RC(check_launch("sg_gather"));
         sg_mark(3);
@@ -1149,9 +1175,9 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
             // previous layer's epilogue), then run the FP8 conv
             quantize_conv_input(m, i, x, B, st);
             CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
-            conv_tc_launch(m->tcplan[i], B, st);
+            conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
         } else if (m->bf16) {
-            conv_tc_launch(m->tcplan[i], B, st);
+            conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
         } else if (m->f32tc[i]) {
             const size_t n = m->conv[i].n_in;
             if (i > 0 && !m->f32tc[i - 1]) {       // the CUDA-core layer before left no maximum
@@ -1179,17 +1205,17 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
     const void *flat_in = x;
     if (d.pool > 1) {
         const Shape s = conv_out(d, d.n_conv);
-        PoolArgs po{x, m->pool_out, B, s.n, m->pool_n, s.c, m->bf16 ? 1 : 0};
+        PoolArgs po{x, m->pool_out, B, s.n, m->pool_n, s.c, m->bf16 ? 1 : 0, early};
         launch_maxpool(po, st);
         RC(check_launch("maxpool"));
         flat_in = m->pool_out;
         map[10] = ei; mark(st);
     }
     DenseArgs da{static_cast<const float *>(flat_in), static_cast<const float *>(m->dense_w), m->dense_b, m->dense_part,
-                 m->cnn_lat, B, d.cnn_dense, m->flat, m->splits, 1};     // (a bf16 model's x and w go to dense_tc)
+                 m->cnn_lat, B, d.cnn_dense, m->flat, m->splits, 1, early};     // (a bf16 model's x and w go to dense_tc)
     if (m->bf16) {
         // tensor cores: split partials, then the same fixed-order reduction
-        dense_tc_launch(m->dense_tc, B, m->dense_part, st);
+        dense_tc_launch(m->dense_tc, B, m->dense_part, early, st);
         da.splits = m->dense_tc_splits;
         launch_dense_reduce(da, st);
     } else {
@@ -1198,7 +1224,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
     if (d.cnn_dense2) {
         // the second CNN dense layer (FP32 on every dtype: a cnn_dense x cnn_dense2 matrix per pose)
         DenseArgs d2{m->cnn_lat, m->dense2_w, m->dense2_b, m->dense_part, m->cnn_lat2, B, d.cnn_dense2, d.cnn_dense,
-                     dense_splits(d.cnn_dense), 1};
+                     dense_splits(d.cnn_dense), 1, early};
         launch_dense(d2, st);
     }
     RC(check_launch("dense"));
@@ -1690,9 +1716,9 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
         // one untimed launch, then three timed back to back
         auto time_plan = [&](ConvTcPlan &pl, float &ms) -> int {
             prepare_input();
-            conv_tc_launch(pl, B, st);
+            conv_tc_launch(pl, B, false, 0, st);
             CU(cudaEventRecord(e0, st));
-            for (int r = 0; r < 3; ++r) conv_tc_launch(pl, B, st);
+            for (int r = 0; r < 3; ++r) conv_tc_launch(pl, B, false, 0, st);
             CU(cudaEventRecord(e1, st));
             CU(cudaStreamSynchronize(st));
             RC(check_launch("autotune conv"));

@@ -19,6 +19,34 @@
 
 namespace fusion {
 
+// Programmatic dependent launch: with `early` a kernel may start while the one before it on the stream still runs, once
+// all of that one's CTAs have called launch_next() or ended; what it reads of the earlier kernels' results, and anything
+// it writes, comes after wait_prior(), which returns when they have completed; such results are read by plain loads
+// (not __ldg: they change within the kernel's lifetime).  Every thread of such a kernel calls wait_prior(), so that a
+// kernel never completes before the ones ahead of it.  A kernel that uses tensor memory calls launch_next() once it holds
+// its own: whatever a waiting CTA holds, the kernels it waits for then need nothing more, on either stream.  Without
+// `early` both calls do nothing.
+// Used where a call's kernels are short and leave most multiprocessors idle (early_launches in capi.cu): a kernel's
+// launch, barrier setup, tensor-memory allocation and weight copies then overlap the one before it.
+__device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <class... P, class... A>
+inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool early,
+                          const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 constexpr int kFeat = 19;
 constexpr int kMaxSupportW = 11;     // 2k+1 for k <= 5
 constexpr int kGridCellsMax = 16;    // graph cell list: at most 16 cells per axis
@@ -87,6 +115,7 @@ struct PoolArgs {
     const void *x; void *y;
     int B, n_in, n_out, c;
     int bf16;
+    bool early;           // see launch_kernel
 };
 void launch_maxpool(const PoolArgs &a, cudaStream_t s);
 
@@ -98,6 +127,7 @@ struct DenseArgs {
     float *y;             // [B][N]
     int B, N, K, splits;
     int relu;
+    bool early;           // see launch_kernel
 };
 void launch_dense(const DenseArgs &a, cudaStream_t s);
 // The same layer on the tensor cores at FP32's accuracy (k_dense_f32tc.cu), with at most a.splits splits; the order of
@@ -120,7 +150,7 @@ struct DenseTcPlan {
 int dense_tc_splits(int K, int N);
 int dense_tc_plan(DenseTcPlan &plan, const void *x, const void *w, int max_poses, int N, int K, unsigned *err,
                   char *why, size_t why_len);
-void dense_tc_launch(DenseTcPlan &plan, int B, float *part, cudaStream_t s);
+void dense_tc_launch(DenseTcPlan &plan, int B, float *part, bool early, cudaStream_t s);
 
 // Tensor-core (tcgen05) BF16 conv: a plan per layer holds the TMA tensor map of
 // the layer's input buffer and the launch geometry.
@@ -177,7 +207,10 @@ struct ConvTcSpec {
 };
 // Build the plan; returns 0, or nonzero with a reason in `why`.
 int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &spec, char *why, size_t why_len);
-void conv_tc_launch(ConvTcPlan &plan, int B, cudaStream_t s);
+// busy_sms: multiprocessors that other kernels are expected to hold, so that the tile height is chosen for the others.
+void conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s);
+// Estimated clocks of the plan's launch for B poses.
+double conv_tc_clocks(const ConvTcPlan &plan, int B);
 // Test of the bounded waits: the plan's next launch issues no loads, so its waits run out (about 1 s)
 // and it sets FUSION_ERR_TIMEOUT; later launches are normal.
 void conv_tc_stall_next(ConvTcPlan &plan);
@@ -300,6 +333,7 @@ struct SgStepArgs {
     int A, H;
     const int32_t *A_dev;  // non-null: the atom count is *A_dev (A is then the launch capacity)
     int nodes_per_warp;    // 1, 2, 4 or 8 (anything else: 4); the results do not depend on it
+    bool early;            // see launch_kernel (launch_sg_message)
 };
 void launch_sg_step(const SgStepArgs &a, cudaStream_t s);
 // The step's messages alone (the sums of sg_step_kernel, same order) into m [A][H].
@@ -319,6 +353,7 @@ struct SgGruTcArgs {
     const int32_t *A_dev;  // non-null: the atom count is *A_dev (A is then the launch capacity)
     unsigned *err;
     int stall;             // test of the bounded waits: no weight copy is issued, so the first wait runs out
+    bool early;            // see launch_kernel
 };
 void launch_sg_gru_tc(const SgGruTcArgs &a, cudaStream_t s);
 // Sets the tensor-core graph kernels' shared-memory limits and sizes their persistent grids (call before
@@ -340,6 +375,7 @@ struct SgStageTcArgs {
     const int32_t *A_dev;
     unsigned *err;
     int stall;             // as SgGruTcArgs::stall
+    bool early;            // see launch_kernel
 };
 void launch_sg_stage_tc(const SgStageTcArgs &a, cudaStream_t s);
 // The gate image: BF16 hi / lo parts of [W_i columns of h ; W_j] ([2H][H]) then of W_i's columns of h0
@@ -360,6 +396,7 @@ struct SgGatherArgs {
     const float *wo_t, *bo;   // [H][G], [G] (linear gather: the only matrix)
     float *out;            // [B][G]
     int B, H, G, gated;
+    bool early;            // see launch_kernel
 };
 void launch_sg_gather(const SgGatherArgs &a, cudaStream_t s);
 

@@ -161,6 +161,8 @@ __global__ void maxpool2_kernel(PoolArgs a) {
     // one thread per (pose, z, y, x, channel group) of the output: 8 bf16 channels (one 16-byte load per
     // source voxel) or 4 float channels
     constexpr int CG = BF16 ? 8 : 4;
+    launch_next();
+    wait_prior();
     const int cq = a.c / CG;
     const long long total = (long long)a.B * a.n_out * a.n_out * a.n_out * cq;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -225,8 +227,8 @@ void launch_maxpool(const PoolArgs &a, cudaStream_t s) {
     long long nb = (total + 255) / 256;
     if (nb > 152LL * 16) nb = 152LL * 16;
     const int blocks = (int)(nb < 1 ? 1 : nb);
-    if (a.bf16) maxpool2_kernel<true><<<blocks, 256, 0, s>>>(a);
-    else maxpool2_kernel<false><<<blocks, 256, 0, s>>>(a);
+    if (a.bf16) launch_kernel(maxpool2_kernel<true>, blocks, 256, 0, s, a.early, a);
+    else launch_kernel(maxpool2_kernel<false>, blocks, 256, 0, s, a.early, a);
 }
 
 }  // namespace fusion

@@ -87,7 +87,7 @@ struct Args {
     int blocked;           // input layout: 0 NDHWC, 1 channel-blocked, 2 parity-split
     Geo g;
     unsigned *err;
-    int *tile_counter;
+    int *tile_counter;     // [0] tiles handed out beyond each CTA's first, [1] CTAs done (both zero between launches)
 };
 
 __device__ __forceinline__ void phase_taps(const Args &a, int ph, int &pz, int &py, int &px, int &nz, int &ny,
@@ -499,6 +499,11 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
     }
     __syncthreads();
     if (warp == 1) tc::tmem_dealloc(tbase, TCOLS);
+    // the last CTA to end resets the counters for the next launch
+    if (tid == 0) {
+        __threadfence();
+        if (atomicInc(reinterpret_cast<unsigned *>(a.tile_counter + 1), gridDim.x - 1) == gridDim.x - 1) a.tile_counter[0] = 0;
+    }
 }
 
 // ---- the two FP16 parts of a map -------------------------------------------
@@ -737,7 +742,8 @@ int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &sp, char *why, siz
         snprintf(why, why_len, "no tile fits shared memory");
         return -1;
     }
-    if (!P.counter && cudaMalloc(&P.counter, sizeof(int)) != cudaSuccess) {
+    if (!P.counter && (cudaMalloc(&P.counter, 2 * sizeof(int)) != cudaSuccess ||
+                       cudaMemset(P.counter, 0, 2 * sizeof(int)) != cudaSuccess)) {
         cudaGetLastError();
         snprintf(why, why_len, "cannot allocate the tile counter");
         return -2;
@@ -753,7 +759,6 @@ static void launch_t(const ConvF32TcPlan::Impl &P, const ConvF32TcPlan::Impl::Va
     cudaFuncSetAttribute(conv3d_f32tc_kernel<NT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)V.smem);
     const unsigned tiles = (unsigned)(V.g.nbx * V.g.nby * V.g.nbz * V.g.nblk) * (unsigned)a.B;
     const unsigned grid = std::min(tiles, (unsigned)P.sms);
-    cudaMemsetAsync(P.counter, 0, sizeof(int), s);
     conv3d_f32tc_kernel<NT, T><<<grid, Roles<NT, T>::THREADS, V.smem, s>>>(V.tmap, a);
 }
 

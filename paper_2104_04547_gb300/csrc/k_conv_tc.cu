@@ -160,7 +160,7 @@ struct Args {
     int res_blocked;            // xres is channel-blocked: [pose][z][y][cres / 8][x][8]
     Geo g;
     unsigned *err;
-    int *tile_counter;          // tiles handed out beyond each CTA's first (zeroed before every launch)
+    int *tile_counter;          // [0] tiles handed out beyond each CTA's first, [1] CTAs done (both zero between launches)
 };
 
 __device__ __forceinline__ void phase_taps(const Args &a, int ph, int &pz, int &py, int &px, int &nz, int &ny,
@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = *tmem_slot;
+    launch_next();            // the tensor memory is held: see launch_kernel
     // the first four epilogue warps (one per tensor-memory lane quarter, warp & 3) zero the accumulators; after
     // that each group is re-zeroed by the epilogue that reads it, so every MMA accumulates
     if (warp >= EPI0 && warp < EPI0 + 4) {
@@ -274,6 +275,7 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
+    wait_prior();
 
     auto fail = [&]() {
         *abort_flag = 1;
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                         const int rstep = 8 * rcc;
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4) {
-                            const uint4 t4 = __ldg(reinterpret_cast<const uint4 *>(rsrc + k4 * rstep));
+                            const uint4 t4 = *reinterpret_cast<const uint4 *>(rsrc + k4 * rstep);
                             const __nv_bfloat162 *hp = reinterpret_cast<const __nv_bfloat162 *>(&t4);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
@@ -584,6 +586,11 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     }
     __syncthreads();
     if (warp == 1) tc::tmem_dealloc(tbase, TCOLS);
+    // the last CTA to end resets the counters for the next launch (a memset per launch took 2 us of a small call's path)
+    if (tid == 0) {
+        __threadfence();
+        if (atomicInc(reinterpret_cast<unsigned *>(a.tile_counter + 1), gridDim.x - 1) == gridDim.x - 1) a.tile_counter[0] = 0;
+    }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -1079,7 +1086,8 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
         return -2;
     }
     P.sms = sms;
-    if (!P.counter && cudaMalloc(&P.counter, sizeof(int)) != cudaSuccess) {
+    if (!P.counter && (cudaMalloc(&P.counter, 2 * sizeof(int)) != cudaSuccess ||
+                       cudaMemset(P.counter, 0, 2 * sizeof(int)) != cudaSuccess)) {
         cudaGetLastError();
         snprintf(why, why_len, "cannot allocate the tile counter");
         return -2;
@@ -1090,53 +1098,52 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
 }
 
 template <int N, int T, bool F8, int G>
-static void launch_t(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
+static void launch_t(ConvTcPlan::Impl &P, int B, bool early, cudaStream_t s) {
     cudaFuncSetAttribute(conv3d_tc_kernel<N, T, F8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
     // persistent: one CTA per multiprocessor (one fits at this shared-memory size); tiles from the counter
     P.args.B = B;
     const unsigned tiles = P.grid * (unsigned)B;
     const unsigned grid = tiles < (unsigned)P.sms ? tiles : (unsigned)P.sms;
-    cudaMemsetAsync(P.counter, 0, sizeof(int), s);
-    conv3d_tc_kernel<N, T, F8, G><<<grid, Roles<N, T, G>::THREADS, P.smem, s>>>(P.tmap, P.args);
+    launch_kernel(conv3d_tc_kernel<N, T, F8, G>, grid, Roles<N, T, G>::THREADS, P.smem, s, early, P.tmap, P.args);
 }
 
 template <int N, int T, bool F8>
-static void launch_g(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
+static void launch_g(ConvTcPlan::Impl &P, int B, bool early, cudaStream_t s) {
     if constexpr (T % 8 == 0 && 8 * N <= 256) {
-        if (P.group == 8) return launch_t<N, T, F8, 8>(P, B, s);
+        if (P.group == 8) return launch_t<N, T, F8, 8>(P, B, early, s);
     }
     if constexpr (T == 6 && 6 * N <= 256) {
-        if (P.group == 6) return launch_t<N, T, F8, 6>(P, B, s);
+        if (P.group == 6) return launch_t<N, T, F8, 6>(P, B, early, s);
     }
     if constexpr (T == 6 && N == 64) {
-        if (P.group == 3) return launch_t<N, T, F8, 3>(P, B, s);
+        if (P.group == 3) return launch_t<N, T, F8, 3>(P, B, early, s);
     }
     if constexpr (T % 4 == 0 && 4 * N <= 256) {
-        if (P.group == 4) return launch_t<N, T, F8, 4>(P, B, s);
+        if (P.group == 4) return launch_t<N, T, F8, 4>(P, B, early, s);
     }
     if constexpr (T % 2 == 0 && T != 6 && 2 * N <= 256) {
-        if (P.group == 2) return launch_t<N, T, F8, 2>(P, B, s);
+        if (P.group == 2) return launch_t<N, T, F8, 2>(P, B, early, s);
     }
-    launch_t<N, T, F8, 1>(P, B, s);
+    launch_t<N, T, F8, 1>(P, B, early, s);
 }
 
 template <bool F8>
-static void launch_n(ConvTcPlan::Impl &P, int B, cudaStream_t s) {
+static void launch_n(ConvTcPlan::Impl &P, int B, bool early, cudaStream_t s) {
     switch (P.N * 16 + P.T) {
-    case 32 * 16 + 2: launch_g<32, 2, F8>(P, B, s); break;
-    case 32 * 16 + 6: launch_g<32, 6, F8>(P, B, s); break;
-    case 64 * 16 + 2: launch_g<64, 2, F8>(P, B, s); break;
-    case 64 * 16 + 6: launch_g<64, 6, F8>(P, B, s); break;
-    case 128 * 16 + 1: launch_g<128, 1, F8>(P, B, s); break;
-    case 256 * 16 + 1: launch_g<256, 1, F8>(P, B, s); break;
-    case 32 * 16 + 4: launch_g<32, 4, F8>(P, B, s); break;
-    case 32 * 16 + 8: launch_g<32, 8, F8>(P, B, s); break;
-    case 32 * 16 + 16: launch_g<32, 16, F8>(P, B, s); break;
-    case 64 * 16 + 4: launch_g<64, 4, F8>(P, B, s); break;
-    case 64 * 16 + 8: launch_g<64, 8, F8>(P, B, s); break;
-    case 128 * 16 + 2: launch_g<128, 2, F8>(P, B, s); break;
-    case 128 * 16 + 4: launch_g<128, 4, F8>(P, B, s); break;
-    default: launch_g<256, 2, F8>(P, B, s); break;
+    case 32 * 16 + 2: launch_g<32, 2, F8>(P, B, early, s); break;
+    case 32 * 16 + 6: launch_g<32, 6, F8>(P, B, early, s); break;
+    case 64 * 16 + 2: launch_g<64, 2, F8>(P, B, early, s); break;
+    case 64 * 16 + 6: launch_g<64, 6, F8>(P, B, early, s); break;
+    case 128 * 16 + 1: launch_g<128, 1, F8>(P, B, early, s); break;
+    case 256 * 16 + 1: launch_g<256, 1, F8>(P, B, early, s); break;
+    case 32 * 16 + 4: launch_g<32, 4, F8>(P, B, early, s); break;
+    case 32 * 16 + 8: launch_g<32, 8, F8>(P, B, early, s); break;
+    case 32 * 16 + 16: launch_g<32, 16, F8>(P, B, early, s); break;
+    case 64 * 16 + 4: launch_g<64, 4, F8>(P, B, early, s); break;
+    case 64 * 16 + 8: launch_g<64, 8, F8>(P, B, early, s); break;
+    case 128 * 16 + 2: launch_g<128, 2, F8>(P, B, early, s); break;
+    case 128 * 16 + 4: launch_g<128, 4, F8>(P, B, early, s); break;
+    default: launch_g<256, 2, F8>(P, B, early, s); break;
     }
 }
 
@@ -1150,19 +1157,36 @@ void conv_tc_describe(const ConvTcPlan &plan, int *T, int *groups_per_stage, int
 
 void conv_tc_stall_next(ConvTcPlan &plan) { plan.impl->args.stall = 1; }
 
-void conv_tc_launch(ConvTcPlan &plan, int B, cudaStream_t s) {
-    ConvTcPlan::Impl &M = *plan.impl;
-    auto schedule = [&](const ConvTcPlan::Impl &p) {        // rounds of tiles over the SMs x a tile's clocks
-        const long long tiles = (long long)p.grid * B;
-        return (double)((tiles + p.sms - 1) / p.sms) * p.tile_clk;
+// The plan (this or one of its smaller tiles) with the shortest schedule on all but busy_sms multiprocessors, and its
+// clocks: rounds of tiles x a tile's clocks.
+static ConvTcPlan::Impl &shortest(const ConvTcPlan &plan, int B, int busy_sms, double &clocks) {
+    auto schedule = [&](const ConvTcPlan::Impl &p) {
+        const long long tiles = (long long)p.grid * B, sms = std::max(1, p.sms - busy_sms);
+        return (double)((tiles + sms - 1) / sms) * p.tile_clk;
     };
-    ConvTcPlan::Impl *best = &M;
-    for (auto &q : M.alts)
-        if (schedule(*q->impl) < 0.97 * schedule(*best)) best = q->impl;
-    best->args.stall = M.args.stall;
-    if (best->f8) launch_n<true>(*best, B, s);
-    else launch_n<false>(*best, B, s);
-    best->args.stall = M.args.stall = 0;   // one launch only
+    ConvTcPlan::Impl *best = plan.impl;
+    clocks = schedule(*best);
+    for (auto &q : plan.impl->alts)
+        if (schedule(*q->impl) < 0.97 * clocks) {
+            best = q->impl;
+            clocks = schedule(*best);
+        }
+    return *best;
+}
+
+double conv_tc_clocks(const ConvTcPlan &plan, int B) {
+    double c;
+    shortest(plan, B, 0, c);
+    return c;
+}
+
+void conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s) {
+    double c;
+    ConvTcPlan::Impl &best = shortest(plan, B, busy_sms, c);
+    best.args.stall = plan.impl->args.stall;
+    if (best.f8) launch_n<true>(best, B, early, s);
+    else launch_n<false>(best, B, early, s);
+    best.args.stall = plan.impl->args.stall = 0;   // one launch only
 }
 
 }  // namespace fusion

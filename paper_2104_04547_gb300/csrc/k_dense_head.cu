@@ -65,6 +65,8 @@ struct StreamTile {
 template <int BT>
 __global__ void __launch_bounds__(kDenseThreads, 2) dense_stream_kernel(DenseArgs a) {
     extern __shared__ __align__(16) float dsm[];
+    launch_next();
+    wait_prior();
     using S = StreamTile<BT>;
     constexpr int LD = S::LD, STAGE = S::STAGE, STAGES = S::STAGES;
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
@@ -131,6 +133,8 @@ struct GemmTile {
 template <int BT>
 __global__ void __launch_bounds__(kDenseThreads, 1) dense_tile_kernel(DenseArgs a) {
     extern __shared__ __align__(16) float dsm[];
+    launch_next();
+    wait_prior();
     using S = GemmTile<BT>;
     constexpr int LD = S::LD, STAGE = S::STAGE, NI = BT / 4;
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
@@ -202,6 +206,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_tile_kernel(DenseArgs 
 // the latency of its loads: one thread per output walked 108 partials in 14 rounds, a warp now holds its 14 in flight.
 __global__ void __launch_bounds__(256) dense_reduce_kernel(DenseArgs a) {
     __shared__ float sums[8][32];
+    launch_next();
+    wait_prior();
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     const int e = blockIdx.x * 32 + lane, tot = a.B * a.N;
     const int per = (a.splits + 7) / 8, lo = q * per, hi = min(a.splits, lo + per);
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(256) dense_reduce_kernel(DenseArgs a) {
         for (int i = lo; i < hi; i += 16) {
             float v[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = i + j < hi ? __ldg(p + (size_t)(i + j) * tot) : 0.f;
+            for (int j = 0; j < 16; ++j) v[j] = i + j < hi ? p[(size_t)(i + j) * tot] : 0.f;
 #pragma unroll
             for (int j = 0; j < 16; ++j) s += v[j];
         }
@@ -368,14 +374,16 @@ template <int BT>
 static void launch_stream(const DenseArgs &a, cudaStream_t s) {
     const size_t ring = (size_t)kDenseWarps * StreamTile<BT>::RING * 4;      // covers the [8][BT][32] sums too
     cudaFuncSetAttribute(dense_stream_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-    dense_stream_kernel<BT><<<dim3((a.N + kStreamRows - 1) / kStreamRows, a.splits), kDenseThreads, ring, s>>>(a);
+    launch_kernel(dense_stream_kernel<BT>, dim3((a.N + kStreamRows - 1) / kStreamRows, a.splits), kDenseThreads, ring, s,
+                  a.early, a);
 }
 
 template <int BT>
 static void launch_tile(const DenseArgs &a, cudaStream_t s) {
     const size_t ring = (size_t)kDenseWarps * GemmTile<BT>::RING * 4;        // covers the [8][BT][64] sums too
     cudaFuncSetAttribute(dense_tile_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-    dense_tile_kernel<BT><<<dim3((a.N + kTileN - 1) / kTileN, a.splits, (a.B + BT - 1) / BT), kDenseThreads, ring, s>>>(a);
+    launch_kernel(dense_tile_kernel<BT>, dim3((a.N + kTileN - 1) / kTileN, a.splits, (a.B + BT - 1) / BT), kDenseThreads,
+                  ring, s, a.early, a);
 }
 
 void launch_dense(const DenseArgs &a, cudaStream_t s) {
@@ -390,7 +398,7 @@ void launch_dense(const DenseArgs &a, cudaStream_t s) {
 
 void launch_dense_reduce(const DenseArgs &a, cudaStream_t s) {
     const int tot = a.B * a.N;
-    dense_reduce_kernel<<<(tot + 31) / 32, 256, 0, s>>>(a);
+    launch_kernel(dense_reduce_kernel, (tot + 31) / 32, 256, 0, s, a.early, a);
 }
 
 void launch_head(const HeadArgs &a, cudaStream_t s) {

@@ -79,8 +79,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_tc_kernel(const __grid_cons
     const int kbeg = split * a.kper;
     const int kend = min(a.K, kbeg + a.kper);
     const int niter = (kend - kbeg + kBK - 1) / kBK;
-    const uint64_t deadline = tc::globaltimer() + kWaitNs;
-
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) { tc::mbar_init(&full[i], 1); tc::mbar_init(&empty[i], 1); }
         tc::mbar_init(acc_full, 1);
@@ -92,6 +90,9 @@ __global__ void __launch_bounds__(kThreads, 1) dense_tc_kernel(const __grid_cons
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = *tmem_slot;
+    launch_next();            // the tensor memory is held: see launch_kernel
+    wait_prior();
+    const uint64_t deadline = tc::globaltimer() + kWaitNs;
     auto fail = [&]() {
         *abort_flag = 1;
         atomicOr(a.err, FUSION_ERR_TIMEOUT);
@@ -250,14 +251,14 @@ int dense_tc_plan(DenseTcPlan &plan, const void *x, const void *w, int max_poses
 }
 
 
-void dense_tc_launch(DenseTcPlan &plan, int B, float *part, cudaStream_t s) {
+void dense_tc_launch(DenseTcPlan &plan, int B, float *part, bool early, cudaStream_t s) {
     DenseTcPlan::Impl &P = *plan.impl;
     P.args.B = B;
     P.args.part = part;
     const size_t sm = (size_t)kStages * kStageBytes + (2 * kStages + 1) * 8 + 16;
     cudaFuncSetAttribute(dense_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     dim3 grid(P.gx, P.splits, (unsigned)((B + kBN - 1) / kBN));
-    dense_tc_kernel<<<grid, kThreads, sm, s>>>(P.tw, P.tx, P.args);
+    launch_kernel(dense_tc_kernel, grid, kThreads, sm, s, early, P.tw, P.tx, P.args);
 }
 
 }  // namespace fusion

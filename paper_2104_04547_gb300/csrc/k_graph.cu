@@ -474,6 +474,7 @@ __device__ __forceinline__ void cluster_sync() {
 
 // One launch: a cluster of kGraphSplit CTAs per pose counts, scans (each CTA the whole pose's degrees) and fills.
 __global__ void __launch_bounds__(kThreads) pair_graph_kernel(GraphArgs a) {
+    launch_next();            // nothing that the next kernel sets up depends on this one
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_tmp[33];
     const int p = blockIdx.x / kGraphSplit, part = blockIdx.x % kGraphSplit;
@@ -519,8 +520,7 @@ void launch_radius_graph(const GraphArgs &a, cudaStream_t s) {
     if (a.most_atoms <= kPairAtoms) {
         const size_t n32 = (size_t)(a.most_atoms + 31) / 32 * 32, coords = 3 * n32 * 4;
         if (split <= 128) {      // up to 16 poses
-            const size_t sm = coords + 2 * (n32 + 1) * 4;
-            cudaFuncSetAttribute(pair_graph_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            const size_t sm = coords + 2 * (n32 + 1) * 4;        // 41 KB at kPairAtoms: within the default limit
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = split;
             cfg.blockDim = kThreads;

@@ -175,14 +175,35 @@ __device__ __forceinline__ void message_sums(const SgStepArgs &a, int lane, int 
                 jl[n] = (q0 + lane < dn) ? a.col[e][bn + q0 + lane] : -1;
             }
             const int nq = min(32, dmax - q0);
+            if constexpr (NP == 1) {
+                // one node per warp (small batches, see launch_sg_message): the latency of the L2 reads is the bound, so
+                // eight neighbours are loaded before their in-order additions
+                for (int q = 0; q < nq; q += 8) {
+                    float t[8][HJ];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int jn = __shfl_sync(0xffffffffu, jl[0], (q + u) & 31);
+#pragma unroll
+                        for (int j = 0; j < HJ; ++j)
+                            t[u][j] = q + u < nq ? T[(size_t)jn * H + lane + 32 * j] : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (q + u < nq) {
+#pragma unroll
+                            for (int j = 0; j < HJ; ++j) m[0][j] += t[u][j];
+                        }
+                }
+            } else {
 #pragma unroll 2
-            for (int q = 0; q < nq; ++q) {
+                for (int q = 0; q < nq; ++q) {
 #pragma unroll
-                for (int n = 0; n < NP; ++n) {
-                    const int jn = __shfl_sync(0xffffffffu, jl[n], q);
-                    if (jn >= 0) {                         // warp-uniform: q0 + q < the node's degree
+                    for (int n = 0; n < NP; ++n) {
+                        const int jn = __shfl_sync(0xffffffffu, jl[n], q);
+                        if (jn >= 0) {                         // warp-uniform: q0 + q < the node's degree
 #pragma unroll
-                        for (int j = 0; j < HJ; ++j) m[n][j] += __ldg(T + (size_t)jn * H + lane + 32 * j);
+                            for (int j = 0; j < HJ; ++j) m[n][j] += T[(size_t)jn * H + lane + 32 * j];
+                        }
                     }
                 }
             }
@@ -191,12 +212,17 @@ __device__ __forceinline__ void message_sums(const SgStepArgs &a, int lane, int 
 }
 
 // The messages alone, written to m_out [A][H] (the tensor-core GRU reads them).
+// (One node per warp runs in blocks of 32 warps: a small batch's messages then sit on few multiprocessors, and the
+// convolutions, whose CTAs need one each to themselves, keep the others.)
+constexpr int message_warps(int np) { return np == 1 ? 32 : kWarps; }
 template <int H, int NP>
-__global__ void __launch_bounds__(kWarps * 32) sg_message_kernel(SgStepArgs a, float *m_out) {
+__global__ void __launch_bounds__(32 * (NP == 1 ? 32 : kWarps)) sg_message_kernel(SgStepArgs a, float *m_out) {
     constexpr int HJ = H / 32;
+    launch_next();
+    wait_prior();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int A = a.A_dev ? *a.A_dev : a.A;
-    const int i0 = (blockIdx.x * kWarps + warp) * NP;
+    const int i0 = (blockIdx.x * (NP == 1 ? 32 : kWarps) + warp) * NP;
     if (i0 >= A) return;
     const int np = min(NP, A - i0);
     float m[NP][HJ];
@@ -312,6 +338,8 @@ template <int H>
 __global__ void __launch_bounds__(kWarps * 32) sg_gather_kernel(SgGatherArgs a) {
     __shared__ float sv[kWarps][kGatherAtoms][2 * H];
     __shared__ float part[kWarps][32];
+    launch_next();
+    wait_prior();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = blockIdx.x;
     const int g = blockIdx.y * 32 + lane;
@@ -389,8 +417,9 @@ void launch_step_np(const SgStepArgs &a, cudaStream_t s) {
 
 template <int H, int NP>
 void launch_message_np(const SgStepArgs &a, float *m, cudaStream_t s) {
-    const int blocks = (a.A + kWarps * NP - 1) / (kWarps * NP);
-    sg_message_kernel<H, NP><<<blocks, kWarps * 32, 0, s>>>(a, m);
+    constexpr int warps = message_warps(NP);
+    const int blocks = (a.A + warps * NP - 1) / (warps * NP);
+    launch_kernel(sg_message_kernel<H, NP>, blocks, warps * 32, 0, s, a.early, a, m);
 }
 
 template <int H>
@@ -440,8 +469,8 @@ void launch_sg_message(const SgStepArgs &a, float *m, cudaStream_t s) {
 
 void launch_sg_gather(const SgGatherArgs &a, cudaStream_t s) {
     const dim3 grid(a.B, (a.G + 31) / 32);
-    if (a.H == 64) sg_gather_kernel<64><<<grid, kWarps * 32, 0, s>>>(a);
-    else sg_gather_kernel<32><<<grid, kWarps * 32, 0, s>>>(a);
+    if (a.H == 64) launch_kernel(sg_gather_kernel<64>, grid, kWarps * 32, 0, s, a.early, a);
+    else launch_kernel(sg_gather_kernel<32>, grid, kWarps * 32, 0, s, a.early, a);
 }
 
 }  // namespace fusion

@@ -39,15 +39,6 @@ constexpr int kTileM = 128;
 constexpr int kThreads = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;   // 1 s
 
-// 32 lanes x 16 columns of 32-bit from tensor memory (this warp's lane quarter).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-
 // Shared-memory plan for width H (bytes).
 template <int H>
 struct Plan {
@@ -92,7 +83,7 @@ __device__ __forceinline__ float tanh_fast(float x) { return 1.f - __fdividef(2.
 template <int C>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[C]) {
     if constexpr (C == 16) {
-        tmem_ld16(taddr, r);
+        tc::tmem_ld16(taddr, r);
     } else {
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -157,6 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_gru_tc_kernel(SgGruTcArgs a) {
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = *tmem_slot;
+    launch_next();            // the tensor memory is held: see launch_kernel
 
     // the stage's weights: W_ih and W_hh always, W_e where the next step's transforms are wanted
     bool w_issued = false, w_ready = false;
@@ -177,6 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_gru_tc_kernel(SgGruTcArgs a) {
         w_issued = true;
     }
 
+    wait_prior();            // the weights (this kernel's own) are on their way; what follows reads the step before
     const uint32_t s0 = tc::smem_u32(smem);
     const uint32_t sMhi = s0 + P::oMhi, sMlo = s0 + P::oMlo, sHhi = s0 + P::oHhi, sHlo = s0 + P::oHlo;
     const int quarter = warp & 3;
@@ -201,8 +194,8 @@ __global__ void __launch_bounds__(kThreads, 1) sg_gru_tc_kernel(SgGruTcArgs a) {
                 const int gi = i0 + r;
                 float4 xm = make_float4(0.f, 0.f, 0.f, 0.f), xh = xm;
                 if (gi < A) {
-                    xm = __ldg(reinterpret_cast<const float4 *>(a.m + (size_t)gi * H) + f4);
-                    xh = __ldg(reinterpret_cast<const float4 *>(a.h_in + (size_t)gi * H) + f4);
+                    xm = reinterpret_cast<const float4 *>(a.m + (size_t)gi * H)[f4];
+                    xh = reinterpret_cast<const float4 *>(a.h_in + (size_t)gi * H)[f4];
                 }
                 const uint32_t o = (uint32_t)(((f4 >> 1) * kTileM + r) * 16 + (f4 & 1) * 8);
                 uint2 hi, lo;
@@ -405,6 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_stage_tc_kernel(SgStageTcArgs 
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = *tmem_slot;
+    launch_next();            // the tensor memory is held: see launch_kernel
 
     bool w_issued = false, w_ready = false;
     if (tid == 0 && (int)blockIdx.x < n_tiles && (gate || any_T) && !a.stall) {
@@ -422,6 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_stage_tc_kernel(SgStageTcArgs 
         w_issued = true;
     }
 
+    wait_prior();            // the weights (this kernel's own) are on their way; what follows reads the step before
     const uint32_t s0 = tc::smem_u32(smem);
     const uint32_t sXhi = s0 + P::oXhi, sXlo = s0 + P::oXlo, sYhi = s0 + P::oYhi, sYlo = s0 + P::oYlo;
     const int quarter = warp & 3;
@@ -448,10 +443,10 @@ __global__ void __launch_bounds__(kThreads, 1) sg_stage_tc_kernel(SgStageTcArgs 
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int o = 4 * f4 + u;
-                        f[u] = o < kFeat ? __ldg(a.feat + (size_t)gi * kFeat + o) : 0.f;
+                        f[u] = o < kFeat ? a.feat[(size_t)gi * kFeat + o] : 0.f;
                     }
                     h0 = make_float4(f[0], f[1], f[2], f[3]);
-                    if (a.h_in) h = __ldg(reinterpret_cast<const float4 *>(a.h_in + (size_t)gi * H) + f4);
+                    if (a.h_in) h = reinterpret_cast<const float4 *>(a.h_in + (size_t)gi * H)[f4];
                 }
                 const float4 x = gate ? h : (a.h_in ? h : h0);
                 const uint32_t o = (uint32_t)(((f4 >> 1) * kTileM + r) * 16 + (f4 & 1) * 8);
@@ -690,20 +685,20 @@ static int persistent_grid(int A, int cap) {
 void launch_sg_gru_tc(const SgGruTcArgs &a, cudaStream_t s) {
     if (a.H == 64) {
         const int g = persistent_grid(a.A, gru_cap<64>());
-        if (g > 0) sg_gru_tc_kernel<64><<<g, kThreads, Plan<64>::kSmem, s>>>(a);
+        if (g > 0) launch_kernel(sg_gru_tc_kernel<64>, g, kThreads, Plan<64>::kSmem, s, a.early, a);
     } else {
         const int g = persistent_grid(a.A, gru_cap<32>());
-        if (g > 0) sg_gru_tc_kernel<32><<<g, kThreads, Plan<32>::kSmem, s>>>(a);
+        if (g > 0) launch_kernel(sg_gru_tc_kernel<32>, g, kThreads, Plan<32>::kSmem, s, a.early, a);
     }
 }
 
 void launch_sg_stage_tc(const SgStageTcArgs &a, cudaStream_t s) {
     if (a.H == 64) {
         const int g = persistent_grid(a.A, stage_cap<64>());
-        if (g > 0) sg_stage_tc_kernel<64><<<g, kThreads, StagePlan<64>::kSmem, s>>>(a);
+        if (g > 0) launch_kernel(sg_stage_tc_kernel<64>, g, kThreads, StagePlan<64>::kSmem, s, a.early, a);
     } else {
         const int g = persistent_grid(a.A, stage_cap<32>());
-        if (g > 0) sg_stage_tc_kernel<32><<<g, kThreads, StagePlan<32>::kSmem, s>>>(a);
+        if (g > 0) launch_kernel(sg_stage_tc_kernel<32>, g, kThreads, StagePlan<32>::kSmem, s, a.early, a);
     }
 }
 

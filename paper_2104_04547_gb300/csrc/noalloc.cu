@@ -80,7 +80,7 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
     if (e != cudaSuccess)
         return noalloc_fail(FUSION_ECUDA, std::string("a CUDA error was pending before this call (nothing launched): ") +
                                               cudaGetErrorString(e));
-    fusion::DenseArgs a{x, w, bias, static_cast<float *>(scratch), y, B, N, K, splits, relu ? 1 : 0};
+    fusion::DenseArgs a{x, w, bias, static_cast<float *>(scratch), y, B, N, K, splits, relu ? 1 : 0, false};
     // up to 8 rows the weight stream bounds either form and the CUDA-core one has less to set up; above that its
     // multiply-adds do (us, CUDA cores / tensor cores: 256 x 221,184 59 / 66 at 8 rows and 88 / 67 at 16, 64 x 16,000
     // 18.5 / 20.5 and 26 / 20.5)

@@ -7,7 +7,7 @@ import pytest
 
 from gpu_common import require_gpu, split_csr
 from oracle import fusion_oracle as O
-from synth import configs, weights
+from synth import configs, poses, weights
 
 pytestmark = pytest.mark.gpu
 
@@ -20,12 +20,11 @@ def _pose(rng, n):
 @pytest.mark.parametrize("sizes", [(1, 2, 31, 32, 33, 63, 65, 255, 256, 257, 700), tuple([40, 9, 129] * 7), (2048,),
                                    (2049, 30)])
 def test_edges(sizes):
-    from synth import poses
     F = require_gpu()
     rng = np.random.default_rng(len(sizes))
     ps = [_pose(rng, n) for n in sizes]
     desc = configs.model("fusion-20grid-ragged")
-    m = F.Model(desc, weights.to_blob(desc, weights.init_weights(desc, 7)), max_poses=len(ps), max_atoms=2560)
+    m = F.Model(desc, weights.to_blob(desc, weights.init_weights(desc, 7)), max_poses=len(ps), max_atoms=2560, keep_stages=True)
     m.score(poses.pack(ps))
     for p, (xyz, _, _) in enumerate(ps):
         g = O.radius_graph(xyz, desc["cut_cov"], desc["cut_nc"])
@@ -38,7 +37,6 @@ def test_edges(sizes):
 @pytest.mark.parametrize("copies", [1, 20])
 def test_capacity(copies):
     """A pose over its edge capacity fails the call in both forms; the model stays usable."""
-    from synth import poses
     F = require_gpu()
     rng = np.random.default_rng(1)
     ok = _pose(rng, 60)

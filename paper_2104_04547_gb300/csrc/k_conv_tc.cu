@@ -105,6 +105,7 @@ namespace {
 
 constexpr int kIssReq = 4;
 constexpr int kMaxHalos = 4; // halo buffers at most
+constexpr int kSlab = 2;     // z planes per slab of a single halo buffer
 constexpr int kRing = 4;     // tile indices the producer publishes ahead of the issuers and the epilogue
 
 // Warp roles of one kernel instance: warp 0 loads, warps 1..NI issue MMAs, then 4 x EPW epilogue warps
@@ -136,6 +137,7 @@ struct Geo {
     int groups_per_stage;  // (ty, tx) offset groups per B stage
     int nbs;               // B stages
     int na;                // A buffers
+    int slabs;             // 0, or pieces of kSlab planes that the single A buffer is loaded and released in
     int chunks;            // 16-channel (FP8: 32-channel) chunks of the input
 };
 
@@ -212,6 +214,44 @@ __device__ __forceinline__ void issue_groups(uint32_t on, uint32_t dt, uint32_t 
     }
 }
 
+// One group of a chunk whose halo comes in slabs, its first and/or last one: waits for each slab ahead of the first plane
+// in it (parity full_par), and releases each slab after its last plane (slab0: this warp's first).  Larger dd read a plane
+// at a smaller u, so dd = 0 reads it last.
+template <int NZ, int N, int G, int DPI, bool F8, class Wait>
+__device__ __forceinline__ bool issue_edge(uint32_t on, uint32_t dt, uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh,
+                                           uint32_t row_zy, bool first, bool last, int slab0, uint64_t *a_empty, Wait wait) {
+    constexpr uint32_t IDESC0 = (F8 ? tc::idesc_e4m3(128, 8) : tc::idesc_bf16(128, 8)) & ~(0x3Fu << 17);
+    static_assert(kSlab == 2, "a slab is an even plane and the next");
+    if constexpr (G % 2 == 0 && NZ % 2 == 1) {
+        uint32_t ad[DPI];
+#pragma unroll
+        for (int dd = 0; dd < DPI; ++dd) ad[dd] = al + (uint32_t)(G * dd) * row_zy;
+#pragma unroll
+        for (int u = 0; u <= NZ + G - 2; ++u) {
+            const int s_lo = u > NZ - 1 ? u - (NZ - 1) : 0;
+            const int s_hi = u < G - 1 ? u : G - 1;
+            const uint32_t idesc = IDESC0 | ((uint32_t)((s_hi - s_lo + 1) * N) >> 3) << 17;
+            if (u % 2 == 0 && first) {
+#pragma unroll
+                for (int dd = 0; dd < DPI; ++dd)
+                    if (!wait(slab0 + (G * dd + u) / 2)) return false;
+                tc::tc_fence_after();
+            }
+#pragma unroll
+            for (int dd = 0; dd < DPI; ++dd) {
+                tc::mma_acc<F8>(on, dt + (uint32_t)((G * dd + s_lo) * N), ad[dd], ah,
+                                bl + (uint32_t)((NZ - 1 - (u - s_lo)) * N), bh, idesc);
+                ad[dd] += row_zy;
+            }
+            if (u % 2 == 1 && last && on) tc::mma_commit(&a_empty[slab0 + u / 2]);
+        }
+        if (last && on)
+            for (int s = (NZ + G - 1) / 2; s <= (G * (DPI - 1) + NZ + G - 2) / 2; ++s) tc::mma_commit(&a_empty[slab0 + s]);
+        return true;
+    }
+    return false;                               // not reached: a plan has slabs for even G and odd NZ only
+}
+
 template <int N, int T, bool F8, int G>
 __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(const __grid_constant__ CUtensorMap tmap, Args a) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -223,13 +263,14 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     constexpr int CPR = F8 ? 16 : 8;      // channels per 16-byte row (one core-matrix column)
     const Geo &g = a.g;
     const uint32_t a_bytes = g.a_bytes;                             // buffer stride
-    const uint32_t a_tx = 2u * (uint32_t)(g.hd * g.hh * g.hw) * 16u;  // bytes the two TMA loads deliver
+    const uint32_t a_tx = 2u * (uint32_t)((g.slabs ? kSlab : g.hd) * g.hh * g.hw) * 16u;  // bytes of a halo's (slab's) loads
     unsigned char *sA = smem;
     unsigned char *sB = smem + g.na * a_bytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(sB + g.nbs * g.stage_bytes);
-    uint64_t *a_full = bars;            // [na]
-    uint64_t *a_empty = bars + g.na;    // [na]
-    uint64_t *b_full = a_empty + g.na;  // [nbs]
+    const int a_bars = g.slabs ? g.slabs : g.na;
+    uint64_t *a_full = bars;            // [na] (or [slabs])
+    uint64_t *a_empty = bars + a_bars;  // [na] (or [slabs])
+    uint64_t *b_full = a_empty + a_bars;    // [nbs]
     uint64_t *b_empty = b_full + g.nbs; // [nbs]
     uint64_t *acc_full = b_empty + g.nbs;   // [UNITS]: the tile's MMAs of the group are complete
     uint64_t *acc_empty = acc_full + UNITS; // [UNITS]: the epilogue has read and re-zeroed the group
@@ -251,7 +292,16 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     };
 
     if (tid == 0) {
-        for (int i = 0; i < g.na; ++i) { tc::mbar_init(&a_full[i], 1); tc::mbar_init(&a_empty[i], NI); }
+        for (int i = 0; i < a_bars; ++i) {
+            int readers = NI;           // of a slab: the issuers whose slice groups read its planes
+            if (g.slabs) {
+                readers = 0;
+                for (int d = 0; d < UNITS; d += DPI)
+                    readers += kSlab * i + kSlab > G * d && kSlab * i <= G * (d + DPI - 1) + a.k + G - 2;
+            }
+            tc::mbar_init(&a_full[i], 1);
+            tc::mbar_init(&a_empty[i], readers);
+        }
         for (int i = 0; i < g.nbs; ++i) { tc::mbar_init(&b_full[i], 1); tc::mbar_init(&b_empty[i], NI); }
         for (int u = 0; u < UNITS; ++u) { tc::mbar_init(&acc_full[u], 1); tc::mbar_init(&acc_empty[u], 4 * EPW); }
         tc::mbar_init(mma_done, NI);
@@ -285,7 +335,7 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     // Tiles: a CTA's first is blockIdx.x; the producer takes each further one from a global counter (so a CTA
     // that started late, its SM still busy with another kernel, takes fewer) and publishes every tile index,
     // then -1, through the ring to the issuers and the epilogue.  Every wait's deadline is re-armed per tile.
-    int prod_ai = 0, prod_bi = 0;
+    int prod_ai = 0, prod_as = 0, prod_bi = 0;      // halos, slabs of the halo under way, weight stages
     if (warp == 0 && lane == 0) {
         // ---------------- producer ----------------
         int &ai = prod_ai, &bi = prod_bi;
@@ -305,40 +355,66 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                 for (int ph = 0; ph < g.nphase && !*abort_flag; ++ph) {
                     int pz, py, px, nz, ny, nx;
                     phase_taps(a, ph, pz, py, px, nz, ny, nx);
-                    const int buf = ai % g.na;
-                    if (!tc::mbar_wait(&a_empty[buf], ((ai / g.na) & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
-                    tc::mbar_expect_tx(&a_full[buf], a_tx);
-                    const int S = a.stride;
-                    if (a.blocked == 2) {
-                        // parity-split input: input coordinate 2 o + p - pad = 2 (o + (p - pad) >> 1) + ((p - pad) & 1),
-                        // so the phase's halo is one plain box of the parity sub-grid (p - pad) & 1 per dimension,
-                        // starting (p - pad) >> 1 voxels from the tile (arithmetic shift: rounds down)
-                        const int qx = px - a.pad, qy = py - a.pad, qz = pz - a.pad;
-                        tc::tma_load_5d(sA + buf * a_bytes, &tmap, &a_full[buf], (x0 + (qx >> 1)) * CPR, 2 * c,
-                                        y0 + (qy >> 1), z0 + (qz >> 1), b * 8 + (qz & 1) * 4 + (qy & 1) * 2 + (qx & 1));
-                    } else if (a.blocked) {
-                        // buffer [z][y][K half][x][16 bytes]: the chunk's two 16-byte channel blocks in one box
-                        tc::tma_load_5d(sA + buf * a_bytes, &tmap, &a_full[buf], (x0 - a.pad + a.x_shift) * CPR, 2 * c,
-                                        y0 - a.pad, z0 - a.pad, b);
-                    } else {
-                        // buffer [K half][z][y][x][16 bytes]: one box per 16-byte channel block
-                        for (int j = 0; j < 2; ++j)
-                            tc::tma_load_5d(sA + buf * a_bytes + j * g.plane_bytes, &tmap, &a_full[buf], c * 2 * CPR + j * CPR,
-                                            x0 * S + px - a.pad + a.x_shift, y0 * S + py - a.pad, z0 * S + pz - a.pad, b);
-                    }
-                    ++ai;
                     if (a.xpat) nx = a.xt_n[c];
                     const int ngr = nz > 0 ? ny * nx : 0;   // a phase without z taps adds nothing
                     const uint32_t gbytes = (uint32_t)nz * N * 32;
-                    for (int g0 = 0; g0 < ngr; g0 += g.groups_per_stage) {
+                    int g0 = 0;
+                    auto load_weights = [&]() {              // the next stage
                         const int cnt = min(g.groups_per_stage, ngr - g0);
                         const int st = bi % g.nbs;
-                        if (!tc::mbar_wait(&b_empty[st], ((bi / g.nbs) & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
+                        if (!tc::mbar_wait(&b_empty[st], ((bi / g.nbs) & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); return false; }
                         const uint32_t bytes = (uint32_t)cnt * gbytes;
                         tc::mbar_expect_tx(&b_full[st], bytes);
                         tc::bulk_load(sB + st * g.stage_bytes, wc + (size_t)g0 * gbytes, bytes, &b_full[st]);
                         ++bi;
+                        g0 += g.groups_per_stage;
+                        return true;
+                    };
+                    const int S = a.stride;
+                    if (g.slabs) {
+                        // the chunk's first weights ahead of its slabs, which wait for the chunk before
+                        if (ngr > 0 && !load_weights()) break;
+                        for (prod_as = 0; prod_as < g.slabs; ++prod_as) {
+                            const int z = prod_as * kSlab;
+                            if (!tc::mbar_wait(&a_empty[prod_as], (ai & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT)) break;
+                            tc::mbar_expect_tx(&a_full[prod_as], a_tx);
+                            unsigned char *dst = sA + (size_t)z * g.hh * g.ystep * 16;
+                            if (a.blocked)
+                                tc::tma_load_5d(dst, &tmap, &a_full[prod_as], (x0 - a.pad + a.x_shift) * CPR, 2 * c, y0 - a.pad,
+                                                z0 - a.pad + z, b);
+                            else
+                                for (int j = 0; j < 2; ++j)
+                                    tc::tma_load_5d(dst + j * g.plane_bytes, &tmap, &a_full[prod_as], c * 2 * CPR + j * CPR,
+                                                    x0 - a.pad + a.x_shift, y0 - a.pad, z0 - a.pad + z, b);
+                        }
+                        if (prod_as < g.slabs) { fail(); break; }
+                        prod_as = 0;
+                    } else {
+                        const int buf = ai % g.na;
+                        if (!tc::mbar_wait(&a_empty[buf], ((ai / g.na) & 1) ^ 1, deadline, a.err, FUSION_ERR_TIMEOUT)) { fail(); break; }
+                        tc::mbar_expect_tx(&a_full[buf], a_tx);
+                        if (a.blocked == 2) {
+                            // parity-split input: input coordinate 2 o + p - pad = 2 (o + (p - pad) >> 1) + ((p - pad) & 1),
+                            // so the phase's halo is one plain box of the parity sub-grid (p - pad) & 1 per dimension,
+                            // starting (p - pad) >> 1 voxels from the tile (arithmetic shift: rounds down)
+                            const int qx = px - a.pad, qy = py - a.pad, qz = pz - a.pad;
+                            tc::tma_load_5d(sA + buf * a_bytes, &tmap, &a_full[buf], (x0 + (qx >> 1)) * CPR, 2 * c,
+                                            y0 + (qy >> 1), z0 + (qz >> 1), b * 8 + (qz & 1) * 4 + (qy & 1) * 2 + (qx & 1));
+                        } else if (a.blocked) {
+                            // buffer [z][y][K half][x][16 bytes]: the chunk's two 16-byte channel blocks in one box
+                            tc::tma_load_5d(sA + buf * a_bytes, &tmap, &a_full[buf], (x0 - a.pad + a.x_shift) * CPR, 2 * c,
+                                            y0 - a.pad, z0 - a.pad, b);
+                        } else {
+                            // buffer [K half][z][y][x][16 bytes]: one box per 16-byte channel block
+                            for (int j = 0; j < 2; ++j)
+                                tc::tma_load_5d(sA + buf * a_bytes + j * g.plane_bytes, &tmap, &a_full[buf], c * 2 * CPR + j * CPR,
+                                                x0 * S + px - a.pad + a.x_shift, y0 * S + py - a.pad, z0 * S + pz - a.pad, b);
+                        }
                     }
+                    ++ai;
+                    bool loaded = true;
+                    while (g0 < ngr && loaded) loaded = load_weights();
+                    if (!loaded) break;
                     wc += (size_t)ngr * gbytes;
                 }
             }
@@ -374,8 +450,10 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                     int pz, py, px, nz, ny, nx;
                     phase_taps(a, ph, pz, py, px, nz, ny, nx);
                     const int buf = ai % g.na;
-                    ok = wait_all(&a_full[buf], (ai / g.na) & 1, deadline);
+                    if (!g.slabs) ok = wait_all(&a_full[buf], (ai / g.na) & 1, deadline);
                     if (!ok) { fail(); break; }
+                    const int slab0 = G * d0 / kSlab;
+                    auto slab_full = [&](int i) { return wait_all(&a_full[i], ai & 1, deadline); };
                     // descriptors advance by plain integer adds: the start-address field counts 16-byte rows
                     const uint64_t adesc0 = tc::desc_kmajor(tc::smem_u32(sA + buf * a_bytes), g.lbo_a, sbo_a);
                     const uint32_t lbo_b = (uint32_t)nz * N * 16;    // between the two 8-channel halves
@@ -396,25 +474,55 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                         if (!ok) { fail(); break; }
                         tc::tc_fence_after();
                         const uint64_t bdesc = tc::desc_kmajor(tc::smem_u32(sB + st * g.stage_bytes), lbo_b, 128);
-                        const uint32_t bl = (uint32_t)bdesc, bh = (uint32_t)(bdesc >> 32);
+                        uint32_t bl = (uint32_t)bdesc;
+                        const uint32_t bh = (uint32_t)(bdesc >> 32);
+                        auto advance = [&](int n) {              // past n groups
+                            for (int i = 0; i < n; ++i) {
+                                if (++tx == nx) { tx = 0; al += wrap; }
+                                else al += (uint32_t)xstep;
+                            }
+                            bl += (uint32_t)(n * nz * N * 2);
+                        };
+                        auto edge = [&](bool first, bool last) {
+                            switch (nz) {
+                            case 1: return issue_edge<1, N, G, DPI, F8>(on, dt, al, ah, bl, bh, row_zy, first, last, slab0, a_empty, slab_full);
+                            case 3: return issue_edge<3, N, G, DPI, F8>(on, dt, al, ah, bl, bh, row_zy, first, last, slab0, a_empty, slab_full);
+                            case 5: return issue_edge<5, N, G, DPI, F8>(on, dt, al, ah, bl, bh, row_zy, first, last, slab0, a_empty, slab_full);
+                            case 7: return issue_edge<7, N, G, DPI, F8>(on, dt, al, ah, bl, bh, row_zy, first, last, slab0, a_empty, slab_full);
+                            default: return issue_edge<9, N, G, DPI, F8>(on, dt, al, ah, bl, bh, row_zy, first, last, slab0, a_empty, slab_full);
+                            }
+                        };
+                        int mid = cnt;
+                        bool tail = false;
+                        if (g.slabs) {                           // the chunk's first and last groups apart
+                            if (g0 == 0) {
+                                ok = edge(true, ngr == 1);
+                                if (!ok) { fail(); break; }
+                                advance(1);
+                                --mid;
+                            }
+                            tail = mid > 0 && g0 + cnt == ngr;
+                            mid -= tail;
+                        }
                         switch (nz) {     // k and, at stride 2, (k + 1) / 2 and k / 2 for odd k <= 9
-                        case 1: issue_groups<1, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        case 2: issue_groups<2, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        case 3: issue_groups<3, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        case 4: issue_groups<4, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        case 5: issue_groups<5, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        case 7: issue_groups<7, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
-                        default: issue_groups<9, N, G, DPI, F8>(on, dt, al, ah, bl, bh, cnt, tx, nx, xstep, wrap, row_zy); break;
+                        case 1: issue_groups<1, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        case 2: issue_groups<2, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        case 3: issue_groups<3, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        case 4: issue_groups<4, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        case 5: issue_groups<5, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        case 7: issue_groups<7, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        default: issue_groups<9, N, G, DPI, F8>(on, dt, al, ah, bl, bh, mid, tx, nx, xstep, wrap, row_zy); break;
+                        }
+                        advance(mid);
+                        if (tail) {
+                            edge(false, true);
+                            advance(1);
                         }
                         if (on) tc::mma_commit(&b_empty[st]);
-                        for (int i = 0; i < cnt; ++i) {
-                            if (++tx == nx) { tx = 0; al += wrap; }
-                            else al += (uint32_t)xstep;
-                        }
                         if (++st == g.nbs) { st = 0; b_par ^= 1; }
                     }
                     if (!ok) break;
-                    if (on) tc::mma_commit(&a_empty[buf]);
+                    if (on && !g.slabs) tc::mma_commit(&a_empty[buf]);
                     ++ai;
                 }
             }
@@ -575,8 +683,8 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
     if (warp == 0 && lane == 0) {
         // make sure no copy issued by this CTA is still landing in its shared memory
         const uint64_t dl = tc::globaltimer() + 100000000ull;
-        for (int i = 0; i < g.na; ++i) {
-            const int n = prod_ai > i ? (prod_ai - i + g.na - 1) / g.na : 0;
+        for (int i = 0; i < a_bars; ++i) {
+            const int n = g.slabs ? prod_ai + (i < prod_as) : prod_ai > i ? (prod_ai - i + g.na - 1) / g.na : 0;
             if (n > 0 && !tc::mbar_wait(&a_full[i], (n - 1) & 1, dl)) atomicOr(a.err, FUSION_ERR_TIMEOUT);
         }
         for (int i = 0; i < g.nbs; ++i) {
@@ -1006,6 +1114,15 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
     g.na = 1;
     while (g.na < kMaxHalos && (g.na + 1) * a1 + b_total + bar_bytes <= limit) ++g.na;
     P.smem = g.na * a1 + b_total + bar_bytes;
+    g.slabs = 0;
+    if (g.na == 1 && stride == 1 && k % 2 == 1 && group % 2 == 0 && g.hd / kSlab > 1) {
+        // more barriers than four whole halos have
+        const size_t more = (size_t)std::max(0, g.hd / kSlab - kMaxHalos) * 16;
+        if (P.smem + more <= limit) {
+            g.slabs = g.hd / kSlab;
+            P.smem += more;
+        }
+    }
     if (P.smem > limit) {
         snprintf(why, why_len, "tensor-core conv tile needs %zu bytes of shared memory", P.smem);
         return -1;
@@ -1025,8 +1142,9 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
     const cuuint64_t cpr = (cuuint64_t)(16 / sp.elem);              // elements per 16-byte channel block
     cuuint64_t dims[5] = {(cuuint64_t)sp.cin_pad, nx_in, n, n, (cuuint64_t)sp.max_poses};
     cuuint64_t strides[4] = {rowb, rowb * nx_in, rowb * nx_in * n, rowb * nx_in * n * n};
+    const int box_z = g.slabs ? kSlab : g.hd;
     cuuint32_t box[5] = {(cuuint32_t)cpr, (cuuint32_t)(g.hw * stride), (cuuint32_t)(g.hh * stride),
-                         (cuuint32_t)(g.hd * stride), 1};
+                         (cuuint32_t)(box_z * stride), 1};
     cuuint32_t estr[5] = {1, (cuuint32_t)stride, (cuuint32_t)stride, (cuuint32_t)stride, 1};
     if (sp.blocked == 2) {
         // parity-split: dims (x' * cpr + channel in block, block, y', z', pose * 8 + parity), x' y' z' < n / 2;
@@ -1041,7 +1159,7 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
         const cuuint64_t blocks = (cuuint64_t)sp.cin_pad / cpr;
         dims[0] = nx_in * cpr; dims[1] = blocks; dims[2] = n; dims[3] = n; dims[4] = (cuuint64_t)sp.max_poses;
         strides[0] = nx_in * 16; strides[1] = blocks * nx_in * 16; strides[2] = strides[1] * n; strides[3] = strides[2] * n;
-        box[0] = (cuuint32_t)(g.hw * cpr); box[1] = 2; box[2] = (cuuint32_t)g.hh; box[3] = (cuuint32_t)g.hd; box[4] = 1;
+        box[0] = (cuuint32_t)(g.hw * cpr); box[1] = 2; box[2] = (cuuint32_t)g.hh; box[3] = (cuuint32_t)box_z; box[4] = 1;
     }
     CUresult r = enc(&P.tmap, sp.elem == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 5,
                      const_cast<void *>(sp.x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

@@ -66,6 +66,10 @@
 // multiplies the FP32 accumulator by both, and records the per-pose maximum
 // |output| so the next layer's input can be quantized with its own scale.
 //
+// Halos: up to four buffers where they fit; where only one does, it is loaded and handed back in slabs of two z planes, a
+// barrier pair each.  The chunk's last (ty, tx) group commits a slab as its MMAs pass it and the next chunk's (or tile's)
+// first group waits for each slab as it gets there (issue_edge), so that the load overlaps both.
+//
 // Persistent schedule: one CTA per multiprocessor (the tile's shared memory
 // allows one); a CTA's first tile is its block index and the producer takes
 // each further one from a global counter, passing the index on to the other
@@ -963,7 +967,9 @@ static double tile_clocks(const Args &A, int N, int T, int group) {
             }
             const double halo = g.a_bytes / 36.0 + 500;
             const double mma = std::max(per_group * (T / group), nz * N * 32 / 20.0) * ny * nx;
-            clk += g.na == 1 ? mma + halo : std::max(mma, halo);
+            // slabs: the halo's load overlaps the last group of the chunk before and the first of its own
+            const double wait = g.slabs ? std::max(halo - 2 * mma / (ny * nx), 0.25 * halo) : halo;
+            clk += g.na == 1 ? mma + wait : std::max(mma, halo);
         }
     return clk;
 }
@@ -1114,6 +1120,11 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
     g.na = 1;
     while (g.na < kMaxHalos && (g.na + 1) * a1 + b_total + bar_bytes <= limit) ++g.na;
     P.smem = g.na * a1 + b_total + bar_bytes;
+    // a halo that leaves room for no second one comes in slabs of kSlab planes: its load then overlaps the chunk before and
+    // its own first group (64 poses: full-size residual layer 9.3 -> 9.05 ms, paper-final 48^3 residual layer 1036 -> 965
+    // us, first layer 660 -> 612 us).  With room for two, the second buffer hides the load whole.  Needs an even number of
+    // planes and slice groups that start on a slab.  (Taller stages of one slice group with two halos instead, T = 8 and
+    // G = 8 at 32 channels: 1113 us, a single issuing warp.)
     g.slabs = 0;
     if (g.na == 1 && stride == 1 && k % 2 == 1 && group % 2 == 0 && g.hd / kSlab > 1) {
         // more barriers than four whole halos have

@@ -783,6 +783,8 @@ static bool bf16_split_in(const fusion_model *m, int i, bool on) { return m->bf1
 static bool bf16_blocked_in(const fusion_model *m, int i) {
     return m->bf16 && !m->fp8 && i < m->d.n_conv && m->d.conv[i].stride == 1 && (i > 0 || m->grid_fold >= 0);
 }
+// The bf16 grid is channel-blocked: for the first layer that reads it in place, or for the folding FP8 quantizer.
+static bool grid_blocked(const fusion_model *m) { return bf16_blocked_in(m, 0) || m->fp8_fold >= 0; }
 // Layout of conv layer l's bf16 output: 0 NDHWC, 1 channel-blocked, 2 parity-split (with stride-2 inputs
 // split when `split`).
 static int conv_out_blocked(const fusion_model *m, int l, bool split) {
@@ -962,6 +964,7 @@ int fusion_create(const fusion_model_desc *desc, const void *weights, size_t wei
         // (4 + 1 x-offsets per kernel row instead of 7 for one 32-channel chunk 13/32 zero)
         if (m->fp8 && !c0.residual && conv_tc_fold_ok(c0.c_in, m->grid_cx, c0.k, c0.stride, 1))
             m->fp8_fold = c0.k / 2;
+        if (m->fp8_fold >= 0) m->grid_cx = 24;      // its quantizer's input, channel-blocked (grid_blocked)
         // FP32 on the tensor cores: the first layer's FP16 parts are folded as the BF16 grid is
         if (!m->bf16 && !c0.residual && conv_tc_fold_ok(c0.c_in, 32, c0.k, c0.stride, 2)) m->f32_fold = c0.k / 2;
     }
@@ -1155,7 +1158,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
         return FUSION_OK;
     };
     VoxArgs va{off_d, B, d.grid_n, d.support, d.max_atoms, m->grid, m->grid_cx,
-               m->bf16 ? 1 : 0, m->grid_fold, bf16_blocked_in(m, 0) ? 1 : 0, m->cell_row, m->atom_rec,
+               m->bf16 ? 1 : 0, m->grid_fold, grid_blocked(m) ? 1 : 0, m->cell_row, m->atom_rec,
                m->fp8 || m->f32tc[0] ? m->amax : nullptr};
     // FP8 and FP32: voxelize also reduces each pose's max |grid value| (the first layer's input scale)
     if (va.amax) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
@@ -1505,7 +1508,7 @@ int fusion_fetch_stage(fusion_model *m, int32_t stage, int32_t index, void *dst,
         const size_t n3 = (size_t)d.grid_n * d.grid_n * d.grid_n;
         std::vector<float> t;
         RC(copy_as_f32(m, m->grid, (size_t)p * n3 * m->grid_cx, n3 * m->grid_cx, t));
-        if (bf16_blocked_in(m, 0)) t = unblock(t, d.grid_n, m->grid_cx);
+        if (grid_blocked(m)) t = unblock(t, d.grid_n, m->grid_cx);
         float *o = static_cast<float *>(dst);
         // a folded grid holds feature 16 + f of voxel x in slot 16 + 3 p + f of the same voxel
         for (size_t v = 0; v < n3; ++v)

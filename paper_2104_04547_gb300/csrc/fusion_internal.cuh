@@ -269,7 +269,7 @@ void launch_split_f16(const SplitF16Args &a, int B, cudaStream_t s);
 // Per-pose max |x| of FP32 maps (atomic max, zeroed by the caller); per_pose a multiple of 4.
 void launch_amax_f32(const float *x, int B, size_t per_pose, float *amax, cudaStream_t s);
 
-// Per-pose FP8 quantization of the plain bf16 grid [B][n]^3[32] (channels 0..18) into the folded layout
+// Per-pose FP8 quantization of the channel-blocked bf16 grid [B][n][n][3][n][8] (channels 0..18) into the folded layout
 // the first FP8 conv reads, [B][n][n][n + 1][64]: stored voxel j holds channels 0..15 of grid voxels
 // j - 1 and j (slots 0..31), and channels 16..18 of voxels j - 1 - p + s, s = 0 .. 2p (slots 32 + 3 s + f),
 // zero outside the grid and in the unused slots; codes use the per-pose scale of launch_quantize_per_pose.

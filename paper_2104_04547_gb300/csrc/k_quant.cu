@@ -106,72 +106,64 @@ __global__ void quantize_blocked_kernel(const __nv_bfloat16 *x, uint8_t *q, int 
     }
 }
 
-// One CTA per 4 grid rows (b, z, y): the rows' channels 0..18 are loaded with 16-byte reads and
-// quantized into shared memory (codes are the same E4M3(x / s) as quantize_per_pose_kernel gives),
-// then each stored voxel j = 0 .. n of a row is assembled from them, as described at
-// launch_quantize_fold_fp8, and written with 16-byte stores.
+// One CTA per 4 grid rows (b, z, y) of the channel-blocked grid: the rows' channels 0..18 are loaded with 16-byte reads
+// (neighbouring threads take neighbouring voxels of a block) and quantized into shared memory (codes are the same E4M3(x / s)
+// as quantize_per_pose_kernel gives), 16 + 4 bytes per voxel, then each stored voxel j = 0 .. n of a row is assembled from
+// them in whole words, as described at launch_quantize_fold_fp8, and written with 16-byte stores.  Bound by its reads and
+// writes (48 + 64 bytes per voxel; with 64 + 64 and codes moved byte by byte the first FP8 layer of 56 paper-final poses,
+// this pass included, took 596 us, now 557).
 constexpr int kFoldRows = 4;
 
 __global__ void __launch_bounds__(256) quantize_fold_fp8_kernel(const __nv_bfloat16 *g, uint8_t *q, int B, int n,
                                                                  int p, const float *amax, float *scale, int blocked) {
-    extern __shared__ __align__(16) uint8_t s_code[];     // [kFoldRows][n][20] (19 channels + pad)
+    extern __shared__ __align__(16) uint4 s_lo[];         // [kFoldRows][n] codes of channels 0..15
+    uint32_t *s_hi = reinterpret_cast<uint32_t *>(s_lo + kFoldRows * n);   // [kFoldRows][n] of 16..18, and a zero byte
+    __shared__ float s_inv[kFoldRows];
     const int rows = B * n * n;
     const int r0 = (gridDim.x - 1 - blockIdx.x) * kFoldRows;   // last rows first, as in quantize_per_pose_kernel
     const int nr = min(kFoldRows, rows - r0);
     const int nn = n * n;
-    for (int e = threadIdx.x; e < nr * n * 3; e += blockDim.x) {
-        // 8 channels (one 16-byte load) of voxel v of row r; chunks 0, 1 = channels 0..15, 2 = 16..23
-        const int r = e / (n * 3), rem = e - r * n * 3, v = rem / 3, part = rem - v * 3;
-        const int row = r0 + r, b = row / nn;
-        const float am = amax[b];
-        const float inv = 1.f / (am > 0.f ? am / kE4M3Max : 1.f);
-        const uint4 t = reinterpret_cast<const uint4 *>(g + ((size_t)row * n + v) * 32)[part];
+    if (threadIdx.x < nr) {
+        const int row = r0 + threadIdx.x, b = row / nn;
+        const float s = amax[b] > 0.f ? amax[b] / kE4M3Max : 1.f;
+        s_inv[threadIdx.x] = 1.f / s;
+        if (row % nn == 0) scale[b] = s;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nr * 3 * n; e += blockDim.x) {
+        const int k = e / n, v = e - k * n, r = k / 3, part = k - r * 3;    // 8 channels of voxel v of row r
+        const float inv = s_inv[r];
+        const uint4 t = *reinterpret_cast<const uint4 *>(g + (((size_t)(r0 + r) * 3 + part) * n + v) * 8);
         const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&t);
-        uint8_t *dst = s_code + ((size_t)r * n + v) * 20 + part * 8;
+        uint32_t c[4];
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) {
             const float2 f = __bfloat1622float2(h[k2]);
-            const uint16_t c2 = __nv_cvt_float2_to_fp8x2(make_float2(f.x * inv, f.y * inv), __NV_SATFINITE, __NV_E4M3);
-            if (part < 2 || 2 * k2 < 3) dst[2 * k2] = (uint8_t)(c2 & 0xFF);
-            if (part < 2 || 2 * k2 + 1 < 3) dst[2 * k2 + 1] = (uint8_t)(c2 >> 8);
+            c[k2] = __nv_cvt_float2_to_fp8x2(make_float2(f.x * inv, f.y * inv), __NV_SATFINITE, __NV_E4M3);
         }
-    }
-    if (threadIdx.x < nr && (r0 + threadIdx.x) % nn == 0) {
-        const int b = (r0 + threadIdx.x) / nn;
-        scale[b] = amax[b] > 0.f ? amax[b] / kE4M3Max : 1.f;
+        if (part < 2) reinterpret_cast<uint2 *>(s_lo + r * n + v)[part] = make_uint2(c[0] | c[1] << 16, c[2] | c[3] << 16);
+        else s_hi[r * n + v] = c[0] | (c[1] & 0xFFu) << 16;
     }
     __syncthreads();
     const int nx = n + 1;
     for (int e = threadIdx.x; e < nr * nx; e += blockDim.x) {
         const int r = e / nx, j = e - r * nx;
-        const uint8_t *cr = s_code + (size_t)r * n * 20;
-        __align__(16) uint8_t out[64];
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        uint4 out[4];
+        out[0] = j > 0 ? s_lo[r * n + j - 1] : zero;
+        out[1] = j < n ? s_lo[r * n + j] : zero;
+        uint32_t w[7];                                // 2p + 1 <= 7 positions (k <= 7) of three bytes
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int x = j - 1 + h;
-            const bool in = x >= 0 && x < n;
-#pragma unroll
-            for (int c = 0; c < 16; ++c) out[16 * h + c] = in ? cr[x * 20 + c] : 0;
-        }
-#pragma unroll
-        for (int qq = 32; qq < 64; ++qq) out[qq] = 0;
-#pragma unroll
-        for (int sl = 0; sl < 7; ++sl) {              // 2p + 1 <= 7 positions (k <= 7); constant slot indices
+        for (int sl = 0; sl < 7; ++sl) {
             const int x = j - 1 - p + sl;
-            if (sl > 2 * p || x < 0 || x >= n) continue;
-#pragma unroll
-            for (int f = 0; f < 3; ++f) out[32 + 3 * sl + f] = cr[x * 20 + 16 + f];
+            w[sl] = sl <= 2 * p && x >= 0 && x < n ? s_hi[r * n + x] : 0u;
         }
-        if (blocked) {
-            // [row][16-byte block u][x = j][16]
+        out[2] = make_uint4(w[0] | w[1] << 24, w[1] >> 8 | w[2] << 16, w[2] >> 16 | w[3] << 8, w[4] | w[5] << 24);
+        out[3] = make_uint4(w[5] >> 8 | w[6] << 16, w[6] >> 16, 0u, 0u);
+        // [row][16-byte block u][x = j][16], or [row][x = j][64]
+        uint4 *const dst = reinterpret_cast<uint4 *>(q) + (size_t)(r0 + r) * nx * 4;
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                *reinterpret_cast<uint4 *>(q + (((size_t)(r0 + r) * 4 + u) * nx + j) * 16) = reinterpret_cast<const uint4 *>(out)[u];
-        } else {
-            uint4 *dst = reinterpret_cast<uint4 *>(q + ((size_t)(r0 + r) * nx + j) * 64);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) dst[u] = reinterpret_cast<const uint4 *>(out)[u];
-        }
+        for (int u = 0; u < 4; ++u) dst[blocked ? u * nx + j : j * 4 + u] = out[u];
     }
 }
 
@@ -180,7 +172,7 @@ __global__ void __launch_bounds__(256) quantize_fold_fp8_kernel(const __nv_bfloa
 void launch_quantize_fold_fp8(const void *grid_bf16, void *q_fp8, int B, int n, int p, const float *amax,
                               float *scale, int blocked, cudaStream_t s) {
     const int rows = B * n * n;
-    const size_t sm = (size_t)kFoldRows * n * 20;
+    const size_t sm = (size_t)kFoldRows * n * 20;     // at most 7.7 KB (n <= 96)
     quantize_fold_fp8_kernel<<<(unsigned)((rows + kFoldRows - 1) / kFoldRows), 256, sm, s>>>(
         static_cast<const __nv_bfloat16 *>(grid_bf16), static_cast<uint8_t *>(q_fp8), B, n, p, amax, scale, blocked);
 }

@@ -26,7 +26,9 @@
 // no atomics).  A tile with no candidate stores zeros without staging anything.
 //
 // Stores: one contiguous vector per voxel (16-byte stores) in the NDHWC layout
-// (float32, or bf16 for the FP8 path's quantizer) or, for the bf16 tensor-core
+// (float32, or bf16), channel-blocked with 24 channels for the FP8 path's folding
+// quantizer (in NDHWC order at 64 bytes a voxel a store reached one 16-byte piece of
+// each of 32 lines: 186 -> 153 us at 56 poses of 48^3) or, for the bf16 tensor-core
 // conv, channel-blocked with the 3 channels beyond the first 16 folded along x
 // (fold_pad = p >= 0): the second 16-channel chunk of voxel x holds features
 // 16..18 of voxels x - p .. x - p + 4, so that chunk needs 2 x-offsets of a 7^3
@@ -223,11 +225,11 @@ constexpr int kTileZ = 2;                 // z-slices per tile
 constexpr int kStage = 128;               // candidate records staged at a time
 constexpr int kMaxRuns = 32;              // candidate runs per tile: kTileZ + 2k <= 12
 
-// Element offset of 8-channel block c0 / 8 of voxel (z, y, x) of pose p, 32 bf16 channels per voxel:
-// NDHWC, or channel-blocked [p][z][y][4][x][8].
-__device__ __forceinline__ size_t bf16_block_off(int p, int z, int y, int x, int c0, int n, int blocked) {
+// Element offset of 8-channel block c0 / 8 of voxel (z, y, x) of pose p, nb blocks of bf16 channels per voxel:
+// NDHWC, or channel-blocked [p][z][y][nb][x][8].
+__device__ __forceinline__ size_t bf16_block_off(int p, int z, int y, int x, int c0, int n, int nb, int blocked) {
     const size_t row = ((size_t)p * n + z) * n + y;
-    return blocked ? ((row * 4 + c0 / 8) * n + x) * 8 : (row * n + x) * 32 + c0;
+    return blocked ? ((row * nb + c0 / 8) * n + x) * 8 : (row * n + x) * (nb * 8) + c0;
 }
 
 // BPW: x-boxes per warp (a tile spans whole x-rows: ceil(n / 4) boxes; warp w takes boxes w, w + 6, ..., so
@@ -241,6 +243,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
     const int WP = atom_rec_wpad(K), RECF = atom_rec_floats(K);
     const int RW = WP + 20;                            // staged floats per record (weights + features)
     const int nxb = (n + 3) / 4;                       // x-boxes of a row
+    const int nb = a.cx / 8;                           // bf16: 8-channel blocks per voxel (3, or 4)
     const int tiles_y = (n + kTileY - 1) / kTileY;
     const int t = blockIdx.x, p = blockIdx.y;
     const int y0 = (t % tiles_y) * kTileY, z0 = (t / tiles_y) * kTileZ;
@@ -293,8 +296,9 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
                 __nv_bfloat16 *const out = reinterpret_cast<__nv_bfloat16 *>(a.out);
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
-                    *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 8 * b, n, a.blocked)) =
-                        make_uint4(0u, 0u, 0u, 0u);
+                    if (b < nb)
+                        *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 8 * b, n, nb, a.blocked)) =
+                            make_uint4(0u, 0u, 0u, 0u);
             } else {
                 float4 *out = reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.out) +
                                                          ((((size_t)p * n + vz) * n + vy) * n + vx) * CX);
@@ -400,7 +404,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
             if (in) {
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    if (fold && b >= 2) break;         // folded: blocks 2 and 3 after the fold below
+                    if (b >= nb || (fold && b >= 2)) break;      // folded: blocks 2 and 3 after the fold below
                     __align__(16) __nv_bfloat16 v8[8];
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
@@ -408,7 +412,7 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
                         v8[q] = __float2bfloat16_rn(c < kFeat ? acc[c < kFeat ? c : 0] : 0.f);
                         if (AMAX) vmax = fmaxf(vmax, fabsf(__bfloat162float(v8[q])));
                     }
-                    *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 8 * b, n, a.blocked)) =
+                    *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 8 * b, n, nb, a.blocked)) =
                         *reinterpret_cast<const uint4 *>(v8);
                 }
             }
@@ -457,9 +461,9 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
                 for (int f = 0; f < 3; ++f) v16[3 * sl + f] = ok ? h[xs * 3 + f] : __float2bfloat16_rn(0.f);
             }
             v16[15] = __float2bfloat16_rn(0.f);
-            *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 16, n, a.blocked)) =
+            *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 16, n, nb, a.blocked)) =
                 reinterpret_cast<const uint4 *>(v16)[0];
-            *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 24, n, a.blocked)) =
+            *reinterpret_cast<uint4 *>(out + bf16_block_off(p, vz, vy, vx, 24, n, nb, a.blocked)) =
                 reinterpret_cast<const uint4 *>(v16)[1];
         }
     }

@@ -633,7 +633,6 @@ __global__ void __launch_bounds__(Roles<N, T, G>::THREADS, 1) conv3d_tc_kernel(c
                         v[j] = __float_as_uint(fmaxf(t + a.bias[cc + j], 0.f));
                     }
                     if (a.residual) {
-                        // the input is read-only for the whole launch (the output is another buffer)
                         // 8-channel blocks k4 = 0..3: contiguous (NDHWC) or n_out voxels apart (blocked)
                         const __nv_bfloat16 *rsrc = a.xres + rbase + zz * zstep_r + (size_t)cc * rcc;
                         const int rstep = 8 * rcc;
@@ -1121,10 +1120,10 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
     while (g.na < kMaxHalos && (g.na + 1) * a1 + b_total + bar_bytes <= limit) ++g.na;
     P.smem = g.na * a1 + b_total + bar_bytes;
     // a halo that leaves room for no second one comes in slabs of kSlab planes: its load then overlaps the chunk before and
-    // its own first group (64 poses: full-size residual layer 9.3 -> 9.05 ms, paper-final 48^3 residual layer 1036 -> 965
-    // us, first layer 660 -> 612 us).  With room for two, the second buffer hides the load whole.  Needs an even number of
-    // planes and slice groups that start on a slab.  (Taller stages of one slice group with two halos instead, T = 8 and
-    // G = 8 at 32 channels: 1113 us, a single issuing warp.)
+    // its own first group (64 poses: full-size residual layer 9.33 -> 9.12 ms, paper-final 48^3 residual layer 1040 ->
+    // 961 us, first layer 704 -> 618 us).  With room for two, the second buffer hides the load whole.  Needs an even number of
+    // planes and slice groups that start on a slab.  (A tile of one slice group with two halos and two accumulator sets
+    // instead, T = 8 and G = 8 at 32 channels: 1113 us, a single issuing warp.)
     g.slabs = 0;
     if (g.na == 1 && stride == 1 && k % 2 == 1 && group % 2 == 0 && g.hd / kSlab > 1) {
         // more barriers than four whole halos have

@@ -51,12 +51,12 @@ CONV_TRAFFIC = {
 
 # DRAM bytes of one voxelize launch at 64 poses (ncu dram__bytes_read.sum + dram__bytes_write.sum), valid for the
 # voxelize source they were taken on (sha256 prefix as for the conv); otherwise null.
-# Taken on 32 poses (171.96 MB = 3.46 MB read + 168.50 MB written) and scaled x2: the grid and the records scale
+# Taken on 32 poses (171.50 MB = 3.46 MB read + 168.04 MB written) and scaled x2: the grid and the records scale
 # with the pose count.  Part of a launch's writes can still sit in L2 when it ends, so this undercounts slightly.
 VOX_TRAFFIC = {
-    "src": "d333f95110c47935",
+    "src": "78415aeadf2a5dbd",
     "poses": 64,
-    "bf16": 2 * 171.96e6,
+    "bf16": 2 * 171.50e6,
 }
 
 

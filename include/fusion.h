@@ -264,9 +264,13 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value);
  * fastest tile configuration (output slices per CTA, output slices per MMA,
  * kernel-offset groups per weight stage, weight stages) by timing
  * every configuration that fits shared memory on the given batch (scored once
- * first); the sweep's winner replaces the layer's default only if, timed
- * against it three more times in alternation, its best time is at least 2%
- * under the default's.  Then the graph convolution's nodes per warp (1, 2, 4, 8) by timing
+ * first), among them the smaller tiles that small batches may take; the
+ * sweep's winner replaces the tile that a call of this batch size takes by
+ * default only if, timed against it three more times in alternation, its best
+ * time is at least 2% under, and the layers' winners stay only if whole calls
+ * with them are faster than with the defaults.  Calls of this batch size then
+ * take the winners; those of other sizes choose between them (or the default,
+ * where a smaller tile won) and the smaller tiles by their estimated times.  Then the graph convolution's nodes per warp (1, 2, 4, 8) by timing
  * whole scoring calls of the batch, since that branch runs beside the
  * convolutions.  Every configuration sums each output in the same order, so
  * the scores do not change.  Replaces the layer plans and the graph schedule;
@@ -285,6 +289,14 @@ int fusion_graph_schedule(fusion_model *m, int32_t *nodes_per_warp);
  * results), unless FUSION_OPT_CONV_SLICES_PER_MMA fixes the layers' tiles.
  * FUSION_EUNSUPPORTED on the FP32 path. */
 int fusion_describe_conv(fusion_model *m, int32_t layer, int32_t *out5);
+
+/* Tile that conv `layer` took in the last fusion_score call (with CUDA graphs: in the
+ * call that captured last): out4 = {output slices per CTA, adjacent output slices
+ * each MMA serves, pieces that its one input halo is loaded in (0: whole halos),
+ * output channels per CTA}.  All zero: the layer ran on the CUDA cores, as an FP32
+ * model's does where no tile fits its shape, or where the model found no device
+ * memory for what the tensor cores need.  FUSION_EINVAL before the first call. */
+int fusion_last_conv_tile(fusion_model *m, int32_t layer, int32_t *out4);
 
 /* ---- aggregation ----
  * The paper ranks compounds by their strongest predicted affinity over all of

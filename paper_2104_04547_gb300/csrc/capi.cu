@@ -316,6 +316,7 @@ struct fusion_model {
     bool last_split2 = true;                      // the conv maps' layout of the last call
     std::vector<int32_t> last_off, last_nlig;
     const void *last_conv_out[FUSION_MAX_CONV] = {};
+    ConvTile last_tile[FUSION_MAX_CONV] = {};     // all zero: on the CUDA cores
     const float *last_h = nullptr;
     float last_ms[17] = {};
     int ev_map[16] = {};
@@ -1178,9 +1179,9 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
             // previous layer's epilogue), then run the FP8 conv
             quantize_conv_input(m, i, x, B, st);
             CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
-            conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
+            m->last_tile[i] = conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
         } else if (m->bf16) {
-            conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
+            m->last_tile[i] = conv_tc_launch(m->tcplan[i], B, early, busy_sms, st);
         } else if (m->f32tc[i]) {
             const size_t n = m->conv[i].n_in;
             if (i > 0 && !m->f32tc[i - 1]) {       // the CUDA-core layer before left no maximum
@@ -1193,7 +1194,7 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
             launch_split_f16(sa, B, st);
             const bool next = i + 1 < d.n_conv && m->f32tc[i + 1];
             if (next) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
-            conv_f32tc_launch(m->f32plan[i], B, next ? m->amax : nullptr, st);
+            m->last_tile[i] = conv_f32tc_launch(m->f32plan[i], B, next ? m->amax : nullptr, st);
         } else {
             ConvArgs ca{static_cast<const float *>(x), static_cast<const float *>(m->conv[i].w), m->conv[i].b,
                         static_cast<float *>(m->act[i]), B, m->conv[i].n_in, m->conv[i].n_out,
@@ -1683,6 +1684,17 @@ int fusion_describe_conv(fusion_model *m, int32_t layer, int32_t *out5) {
     return FUSION_OK;
 }
 
+int fusion_last_conv_tile(fusion_model *m, int32_t layer, int32_t *out4) {
+    if (!m || !out4 || layer < 0 || layer >= m->d.n_conv) return fail(FUSION_EINVAL, "bad arguments");
+    if (m->last_B == 0) return fail(FUSION_EINVAL, "no scoring call yet");
+    const ConvTile &t = m->last_tile[layer];
+    out4[0] = t.slices;
+    out4[1] = t.per_mma;
+    out4[2] = t.slabs;
+    out4[3] = t.channels;
+    return FUSION_OK;
+}
+
 int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses) {
     if (!m || !poses) return fail(FUSION_EINVAL, "NULL argument");
     if (!m->bf16) return fail(FUSION_EUNSUPPORTED, "autotuning applies to the tensor-core (bf16 / fp8) paths");
@@ -1701,6 +1713,42 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
     const int B = n_poses;
     cudaStream_t st = m->stream;
     cudaEvent_t e0 = m->ev[16], e1 = m->ev[17];
+    // the default tiles are what everything is measured against; without a change they stay
+    std::vector<ConvTcSpec> specs(d.n_conv);
+    std::vector<int> tiles(d.n_conv, -1);          // >= 0: the layer takes this tile of a plan of `specs`
+    auto plan_layers = [&](bool tuned) -> int {
+        for (int i = 0; i < d.n_conv; ++i) {
+            const bool win = tuned && tiles[i] >= 0;
+            char why[256] = {0};
+            if (conv_tc_plan(m->tcplan[i], win ? specs[i] : conv_spec(m, i), why, sizeof(why))) return fail(FUSION_ECUDA, why);
+            if (win) conv_tc_tune(m->tcplan[i], B, tiles[i]);
+        }
+        return FUSION_OK;
+    };
+    // whole calls, without graphs (the graph mode is restored at the end, and on an early return with the schedule)
+    struct Restore {
+        fusion_model *m;
+        bool graphs;
+        int npw;
+        ~Restore() {
+            m->use_graph = graphs;
+            m->sg_npw = npw;
+            drop_graphs(m);
+        }
+    } restore{m, m->use_graph, m->sg_npw};
+    m->use_graph = false;
+    auto call_ms = [&](float &ms) -> int {         // median of 5 after one untimed
+        RC(fusion_score(m, poses, n_poses, score_out));
+        std::vector<float> tot;
+        for (int r = 0; r < 5; ++r) {
+            RC(fusion_score(m, poses, n_poses, score_out));
+            tot.push_back(m->last_ms[16]);
+        }
+        std::sort(tot.begin(), tot.end());
+        ms = tot[2];
+        return FUSION_OK;
+    };
+    RC(plan_layers(false));
     for (int i = 0; i < d.n_conv; ++i) {
         const int co = d.conv[i].c_out;
         std::vector<int> Ts = co <= 32   ? std::vector<int>{16, 8, 4}
@@ -1729,16 +1777,26 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
             cudaEventElapsedTime(&ms, e0, e1);
             return FUSION_OK;
         };
-        // the layer's default plan (the caller's slices-per-MMA mode, default tiles) is the one to beat
+        // the layer's default plan (the caller's slices-per-MMA mode, default tiles), with the tile that it takes at this
+        // batch size, is the one to beat
         ConvTcPlan def;
         {
             char why[256] = {0};
-            ConvTcSpec sd = conv_spec(m, i);
-            sd.alts = 0;
-            if (conv_tc_plan(def, sd, why, sizeof(why))) return fail(FUSION_ECUDA, why);
+            if (conv_tc_plan(def, conv_spec(m, i), why, sizeof(why))) return fail(FUSION_ECUDA, why);
         }
         float best_ms = 1e30f;
         int best[4] = {0, 0, 0, 0};
+        int best_tile = -1;                        // >= 0: the default plan's tile of that index, else `best`
+        for (int t = 0; t < conv_tc_tiles(def); ++t) {
+            float ms = 0.f;
+            conv_tc_tune(def, B, t);
+            RC(time_plan(def, ms));
+            if (ms < best_ms) {
+                best_ms = ms;
+                best_tile = t;
+            }
+        }
+        conv_tc_tune(def, 0, 0);
         for (int T : Ts)
             for (int group : {8, 4, 2, 1})
             for (int groups : {1, 2, 3, 4, 6})
@@ -1756,24 +1814,25 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
                     RC(time_plan(trial, ms));
                     if (ms < best_ms) {
                         best_ms = ms;
+                        best_tile = -1;
                         best[0] = T;
                         best[1] = groups;
                         best[2] = nbs;
                         best[3] = group;
                     }
                 }
-        if (best[0] == 0) return fail(FUSION_EUNSUPPORTED, "no tile configuration fits layer " + std::to_string(i));
         ConvTcSpec sp = conv_spec(m, i);
-        const int alts = sp.alts;
-        sp.alts = 0;
-        sp.T = best[0];
-        sp.groups_per_stage = best[1];
-        sp.nbs = best[2];
-        sp.group = best[3];
+        if (best_tile < 0) {
+            sp.T = best[0];
+            sp.groups_per_stage = best[1];
+            sp.nbs = best[2];
+            sp.group = best[3];
+        }
         ConvTcPlan cand;
         {
             char why[256] = {0};
             if (conv_tc_plan(cand, sp, why, sizeof(why))) return fail(FUSION_ECUDA, why);
+            conv_tc_tune(cand, B, std::max(best_tile, 0));
         }
         // The sweep's winner among many close configurations is partly noise (measured: picks 2-3% slower
         // than the default on the full-size residual layers): time it against the default three times
@@ -1786,50 +1845,44 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
             RC(time_plan(cand, ms));
             cand_best = std::min(cand_best, ms);
         }
-        ConvTcSpec chosen = cand_best < 0.98f * def_best ? sp : conv_spec(m, i);
-        chosen.alts = alts;
-        char why[256] = {0};
-        if (conv_tc_plan(m->tcplan[i], chosen, why, sizeof(why))) return fail(FUSION_ECUDA, why);
+        if (cand_best < 0.98f * def_best) {
+            specs[i] = sp;
+            tiles[i] = std::max(best_tile, 0);
+        }
     }
-    drop_graphs(m);
+    // The winners were measured alone.  In a call the graph branch holds some of the multiprocessors (two winners made a
+    // 12-pose paper-final FP8 call 3% slower), so they stay only if whole calls, in alternation, are faster.  They are then
+    // what calls of this batch size take; other sizes choose between a layer's tile and the smaller ones by the estimate
+    // (conv_tc_launch), as the default does.
+    if (*std::max_element(tiles.begin(), tiles.end()) >= 0) {
+        float def_best = 1e30f, tuned_best = 1e30f;
+        for (int r = 0; r < 3; ++r) {
+            float ms = 0.f;
+            RC(plan_layers(false));
+            RC(call_ms(ms));
+            def_best = std::min(def_best, ms);
+            RC(plan_layers(true));
+            RC(call_ms(ms));
+            tuned_best = std::min(tuned_best, ms);
+        }
+        if (tuned_best >= def_best) RC(plan_layers(false));
+    }
 
     // graph convolution: nodes per warp, by the whole call's device time (the branch runs beside the
-    // convolutions, so its own kernel time is not what counts); median of 5 calls after one untimed
-    // on an early return (a failed call) the model gets its graph mode and schedule back
-    struct Restore {
-        fusion_model *m;
-        bool graphs;
-        int npw;
-        bool armed = true;
-        ~Restore() {
-            if (!armed) return;
-            m->use_graph = graphs;
-            m->sg_npw = npw;
-        }
-    } restore{m, m->use_graph, m->sg_npw};
-    const bool graphs = m->use_graph;
-    m->use_graph = false;
+    // convolutions, so its own kernel time is not what counts)
     float best_total = 1e30f;
     int best_npw = 4;
     for (int npw : {4, 8, 2, 1}) {
+        float ms = 0.f;
         m->sg_npw = npw;
-        RC(fusion_score(m, poses, n_poses, score_out));
-        std::vector<float> tot;
-        for (int r = 0; r < 5; ++r) {
-            RC(fusion_score(m, poses, n_poses, score_out));
-            tot.push_back(m->last_ms[16]);
-        }
-        std::sort(tot.begin(), tot.end());
-        if (tot[2] < best_total) {
-            best_total = tot[2];
+        RC(call_ms(ms));
+        if (ms < best_total) {
+            best_total = ms;
             best_npw = npw;
         }
     }
-    restore.armed = false;
-    m->sg_npw = best_npw;
+    restore.npw = best_npw;
     m->sg_npw_set = true;
-    m->use_graph = graphs;
-    drop_graphs(m);
     return FUSION_OK;
 }
 

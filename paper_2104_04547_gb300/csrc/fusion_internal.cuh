@@ -152,6 +152,11 @@ int dense_tc_plan(DenseTcPlan &plan, const void *x, const void *w, int max_poses
                   char *why, size_t why_len);
 void dense_tc_launch(DenseTcPlan &plan, int B, float *part, bool early, cudaStream_t s);
 
+// Tile of a convolution launch (fusion_last_conv_tile).
+struct ConvTile {
+    int slices, per_mma, slabs, channels;
+};
+
 // Tensor-core (tcgen05) BF16 conv: a plan per layer holds the TMA tensor map of
 // the layer's input buffer and the launch geometry.
 struct ConvTcPlan {
@@ -208,7 +213,12 @@ struct ConvTcSpec {
 // Build the plan; returns 0, or nonzero with a reason in `why`.
 int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &spec, char *why, size_t why_len);
 // busy_sms: multiprocessors that other kernels are expected to hold, so that the tile height is chosen for the others.
-void conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s);
+// Returns the tile.
+ConvTile conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s);
+// Tiles that a plan may take (the planned one, then the smaller ones), and the choice of one for calls of B poses in place
+// of the estimate (B = 0: of none, -1: of any); planning anew drops the choice.
+int conv_tc_tiles(const ConvTcPlan &plan);
+void conv_tc_tune(ConvTcPlan &plan, int B, int tile);
 // Estimated clocks of the plan's launch for B poses.
 double conv_tc_clocks(const ConvTcPlan &plan, int B);
 // Test of the bounded waits: the plan's next launch issues no loads, so its waits run out (about 1 s)
@@ -245,8 +255,8 @@ struct ConvF32TcSpec {
 };
 // 0, or nonzero with a reason: the caller then uses launch_conv3d_f32.
 int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &spec, char *why, size_t why_len);
-// amax: per-pose max |output| (atomic max, zeroed by the caller), or null.
-void conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s);
+// amax: per-pose max |output| (atomic max, zeroed by the caller), or null.  Returns the tile.
+ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s);
 // Output channels per tile (0: c_out is not a multiple of 32).
 int conv_f32tc_block(int c_out);
 // Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two; inv_sw[co] = 1 / s_w[co].  Per block of

@@ -762,7 +762,7 @@ static void launch_t(const ConvF32TcPlan::Impl &P, const ConvF32TcPlan::Impl::Va
     conv3d_f32tc_kernel<NT, T><<<grid, Roles<NT, T>::THREADS, V.smem, s>>>(V.tmap, a);
 }
 
-void conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s) {
+ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s) {
     const ConvF32TcPlan::Impl &P = *plan.impl;
     // the tile with the shortest schedule: rounds of tiles over the SMs x a tile's MMA clocks
     int best = 0;
@@ -786,6 +786,7 @@ void conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream
     case 64 * 16 + 2: launch_t<64, 2>(P, V, a, s); break;
     default: launch_t<128, 2>(P, V, a, s); break;
     }
+    return {V.T, 1, 0, P.NT};
 }
 
 void launch_split_f16(const SplitF16Args &a, int B, cudaStream_t s) {

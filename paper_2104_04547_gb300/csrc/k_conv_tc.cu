@@ -732,6 +732,7 @@ struct ConvTcPlan::Impl {
     unsigned grid = 0;
     double tile_clk = 0;    // estimated clocks of a tile, for choosing between tile heights
     std::vector<std::unique_ptr<ConvTcPlan>> alts;   // plans of smaller tiles
+    int tuned_B = 0, tuned = 0;                      // see conv_tc_tune (tile 0 is this plan's, i alts[i - 1]'s)
 };
 
 ConvTcPlan::ConvTcPlan() : impl(new Impl()) {}
@@ -978,6 +979,7 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
 int conv_tc_plan(ConvTcPlan &plan, const ConvTcSpec &sp, char *why, size_t why_len) {
     ConvTcPlan::Impl &P = *plan.impl;
     P.alts.clear();
+    P.tuned_B = 0;
     int r = -1;
     if (sp.T <= 0 && sp.stride == 1 && wide_tiles_ok(sp.c_out, sp.n_out)) {
         ConvTcSpec wide = sp;
@@ -1285,14 +1287,26 @@ void conv_tc_describe(const ConvTcPlan &plan, int *T, int *groups_per_stage, int
 
 void conv_tc_stall_next(ConvTcPlan &plan) { plan.impl->args.stall = 1; }
 
+int conv_tc_tiles(const ConvTcPlan &plan) { return 1 + (int)plan.impl->alts.size(); }
+
+void conv_tc_tune(ConvTcPlan &plan, int B, int tile) {
+    plan.impl->tuned_B = B;
+    plan.impl->tuned = tile;
+}
+
 // The plan (this or one of its smaller tiles) with the shortest schedule on all but busy_sms multiprocessors, and its
-// clocks: rounds of tiles x a tile's clocks.
+// clocks: rounds of tiles x a tile's clocks.  A batch size that a tile was tuned for takes that one.
 static ConvTcPlan::Impl &shortest(const ConvTcPlan &plan, int B, int busy_sms, double &clocks) {
     auto schedule = [&](const ConvTcPlan::Impl &p) {
         const long long tiles = (long long)p.grid * B, sms = std::max(1, p.sms - busy_sms);
         return (double)((tiles + sms - 1) / sms) * p.tile_clk;
     };
     ConvTcPlan::Impl *best = plan.impl;
+    if (B == plan.impl->tuned_B || plan.impl->tuned_B < 0) {
+        if (plan.impl->tuned > 0) best = plan.impl->alts[plan.impl->tuned - 1]->impl;
+        clocks = schedule(*best);
+        return *best;
+    }
     clocks = schedule(*best);
     for (auto &q : plan.impl->alts)
         if (schedule(*q->impl) < 0.97 * clocks) {
@@ -1308,13 +1322,14 @@ double conv_tc_clocks(const ConvTcPlan &plan, int B) {
     return c;
 }
 
-void conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s) {
+ConvTile conv_tc_launch(ConvTcPlan &plan, int B, bool early, int busy_sms, cudaStream_t s) {
     double c;
     ConvTcPlan::Impl &best = shortest(plan, B, busy_sms, c);
     best.args.stall = plan.impl->args.stall;
     if (best.f8) launch_n<true>(best, B, early, s);
     else launch_n<false>(best, B, early, s);
     best.args.stall = plan.impl->args.stall = 0;   // one launch only
+    return {best.T, best.group, best.args.g.slabs, best.N};
 }
 
 }  // namespace fusion

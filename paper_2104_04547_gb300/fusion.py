@@ -51,7 +51,7 @@ EXPORTED = ["fusion_weights_bytes", "fusion_create", "fusion_score", "fusion_des
             "fusion_stage_bytes", "fusion_fetch_stage", "fusion_last_timings", "fusion_cnn_dense_noalloc",
             "fusion_server_create", "fusion_server_submit", "fusion_server_submit_dtype", "fusion_server_poll", "fusion_server_drain",
             "fusion_server_get_stats", "fusion_server_destroy", "fusion_set_option", "fusion_autotune",
-            "fusion_describe_conv", "fusion_best_per_compound", "fusion_graph_schedule"]
+            "fusion_describe_conv", "fusion_last_conv_tile", "fusion_best_per_compound", "fusion_graph_schedule"]
 
 FUSION_NOALLOC_MAX_PARTIALS = 1 << 21
 
@@ -143,6 +143,8 @@ def _load():
     lib.fusion_autotune.restype = C.c_int
     lib.fusion_describe_conv.argtypes = [C.c_void_p, C.c_int32, P(C.c_int32)]
     lib.fusion_describe_conv.restype = C.c_int
+    lib.fusion_last_conv_tile.argtypes = [C.c_void_p, C.c_int32, P(C.c_int32)]
+    lib.fusion_last_conv_tile.restype = C.c_int
     lib.fusion_best_per_compound.argtypes = [P(C.c_float), P(C.c_int32), C.c_int32, C.c_int32, P(C.c_float),
                                              P(C.c_int32)]
     lib.fusion_best_per_compound.restype = C.c_int
@@ -288,6 +290,12 @@ def fusion_describe_conv(model, layer: int) -> dict:
             "slices_per_mma": out[4]}
 
 
+def fusion_last_conv_tile(model, layer: int) -> dict:
+    out = (C.c_int32 * 4)()
+    _check(lib.fusion_last_conv_tile(model, layer, out))
+    return {"slices_per_cta": out[0], "slices_per_mma": out[1], "halo_slabs": out[2], "channels_per_cta": out[3]}
+
+
 def fusion_graph_schedule(model) -> int:
     npw = C.c_int32(0)
     _check(lib.fusion_graph_schedule(model, C.byref(npw)))
@@ -400,6 +408,10 @@ class Model:
 
     def conv_tiles(self):
         return [fusion_describe_conv(self.handle, i) for i in range(self.desc.n_conv)]
+
+    def last_conv_tiles(self):
+        """The tiles of the last score() call's convolutions (all zero: a layer on the CUDA cores)."""
+        return [fusion_last_conv_tile(self.handle, i) for i in range(self.desc.n_conv)]
 
     def graph_nodes_per_warp(self, value=None):
         """Set (1, 2, 4, 8; -1 default) and/or return the graph convolution's nodes per warp."""

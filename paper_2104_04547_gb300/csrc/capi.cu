@@ -303,7 +303,8 @@ struct fusion_model {
     int group_mode = -1;                          // conv output slices per MMA: -1 default per layer, or 1, 2, 4
     bool split2 = true;                           // stride-2 layers read a parity-split input where they can
     int sg_npw = 4;                               // graph convolution: nodes per warp (1, 2, 4, 8)
-    bool sg_npw_set = false;                      // chosen by the caller or the autotuner (else the default)
+    bool sg_npw_set = false;                      // chosen by the caller
+    int sg_npw_B = 0;                             // the batch size it was tuned for (0: not tuned)
     bool serial_branches = false;                 // both branches on the grid stream, one after the other
     bool sg_tc = false;                           // graph steps' GRU and transforms on the tensor cores
     bool sg_stall_next = false;                   // wait-timeout test: the next call's first graph TC launch stalls
@@ -1116,7 +1117,8 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                 sa.nodes_per_warp = m->sg_npw;
                 if (m->sg_tc) {
                     // a warp per node where the branch is the longer one (see message_sums), unless the schedule was chosen
-                    if (graph_early && !m->sg_npw_set) sa.nodes_per_warp = 1;
+                    // or measured on this batch size
+                    if (graph_early && !m->sg_npw_set && m->sg_npw_B != B) sa.nodes_per_warp = 1;
                     sa.early = graph_early;
                     launch_sg_message(sa, m->mbuf, sgs);
                     RC(check_launch("sg_message"));
@@ -1598,6 +1600,7 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value) {
             return fail(FUSION_EINVAL, "graph nodes per warp must be -1 (default), 1, 2, 4 or 8");
         m->sg_npw = value == -1 ? default_npw(m) : (int)value;
         m->sg_npw_set = value != -1;
+        m->sg_npw_B = 0;
         drop_graphs(m);
         return FUSION_OK;
     case FUSION_OPT_SERIAL_BRANCHES:
@@ -1609,7 +1612,7 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value) {
         if (value != -1 && value != 0 && value != 1)
             return fail(FUSION_EINVAL, "graph tensor cores takes -1 (default), 0 or 1");
         m->sg_tc = value == -1 ? m->bf16 : value != 0;
-        if (!m->sg_npw_set) m->sg_npw = default_npw(m);
+        if (!m->sg_npw_set && !m->sg_npw_B) m->sg_npw = default_npw(m);
         drop_graphs(m);
         return FUSION_OK;
     case FUSION_OPT_CONV_STRIDE2_SPLIT: {
@@ -1729,13 +1732,14 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
     struct Restore {
         fusion_model *m;
         bool graphs;
-        int npw;
+        int npw, npw_B;
         ~Restore() {
             m->use_graph = graphs;
             m->sg_npw = npw;
+            m->sg_npw_B = npw_B;
             drop_graphs(m);
         }
-    } restore{m, m->use_graph, m->sg_npw};
+    } restore{m, m->use_graph, m->sg_npw, m->sg_npw_B};
     m->use_graph = false;
     auto call_ms = [&](float &ms) -> int {         // median of 5 after one untimed
         RC(fusion_score(m, poses, n_poses, score_out));
@@ -1870,6 +1874,7 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
 
     // graph convolution: nodes per warp, by the whole call's device time (the branch runs beside the
     // convolutions, so its own kernel time is not what counts)
+    m->sg_npw_B = B;            // small calls too take the schedule under test
     float best_total = 1e30f;
     int best_npw = 4;
     for (int npw : {4, 8, 2, 1}) {
@@ -1882,7 +1887,7 @@ int fusion_autotune(fusion_model *m, const fusion_poses *poses, int32_t n_poses)
         }
     }
     restore.npw = best_npw;
-    m->sg_npw_set = true;
+    restore.npw_B = B;
     return FUSION_OK;
 }
 

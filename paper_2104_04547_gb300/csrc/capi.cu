@@ -241,6 +241,7 @@ struct fusion_model {
     // weights (device)
     struct ConvW {
         void *w = nullptr;        // f32 [k^3][cx][co], or bf16 in the tensor-core layout
+        void *w_hi = nullptr, *w_both = nullptr;      // FP32 on the tensor cores (conv_f32tc_arrange_weights)
         float *b = nullptr;
         int cx_in = 0, n_in = 0, n_out = 0;
     } conv[FUSION_MAX_CONV];
@@ -255,6 +256,7 @@ struct fusion_model {
     bool f32tc[FUSION_MAX_CONV] = {};
     ConvF32TcPlan f32plan[FUSION_MAX_CONV];
     int f32_fold = -1;                            // first layer reads its input x-folded at this pad, or -1
+    int f32_parts = 0;                            // poses whose FP16 parts qbuf holds (0: every layer on the CUDA cores)
     DenseTcPlan dense_tc;                         // tensor-core CNN dense (bf16 / FP8 models)
     int dense_tc_splits = 0;
     int pool_n = 0, pool_c = 0, flat = 0, splits = 1;
@@ -279,7 +281,7 @@ struct fusion_model {
     int fp8_fold = -1;                            // FP8: first conv reads the folded FP8 grid (this pad), or -1
     void *act[FUSION_MAX_CONV] = {};
     void *pool_out = nullptr;
-    void *qbuf = nullptr;         // FP8 input (FP32: the input's two FP16 parts) of the conv layer being computed
+    void *qbuf = nullptr;         // FP8 input (FP32: the two FP16 parts of f32_parts poses' input) of the layer being computed
     float *amax = nullptr, *qscale = nullptr;   // per-pose max |activation| and scale (FP32: its inverse) [max_poses]
     float *conv_sw[FUSION_MAX_CONV] = {};       // per-output-channel weight scales (FP32: their inverses)
     float *dense_part = nullptr, *cnn_lat = nullptr;
@@ -451,31 +453,19 @@ int f32tc_layout(const fusion_model *m, int i) {
 }
 int f32tc_channels(const fusion_model *m, int i) { return i == 0 ? 32 : m->d.conv[i].c_in; }   // 19 padded to 32
 
-// The tensor-core weights and plan of FP32 layer i, on success in m->f32tc[i] (else the layer stays on the CUDA
-// cores: a kernel size no tile fits, or no room for the parts).
-int plan_f32tc(fusion_model *m, int i, const float *w, float *bias) {
+ConvF32TcSpec f32tc_spec(const fusion_model *m, int i) {
     const fusion_conv_desc &c = m->d.conv[i];
-    const int nt = conv_f32tc_block(c.c_out);
-    if (!m->qbuf || !nt) return FUSION_OK;
-    const int cp = f32tc_channels(m, i), fold = i == 0 && m->f32_fold >= 0 ? 1 : 0;
-    const size_t bytes = conv_tc_weight_bytes(cp, nt, c.k, c.stride, 2, fold) * (c.c_out / nt);
-    std::vector<uint8_t> hi(bytes), both(2 * bytes);
-    std::vector<float> isw(c.c_out);
-    conv_f32tc_arrange_weights(w, c.c_out, c.c_in, cp, c.k, c.stride, fold, hi.data(), both.data(), isw.data());
-    void *d_hi = nullptr, *d_both = nullptr;
-    RC_INNER(upload_raw(m, &d_hi, hi.data(), bytes));
-    RC_INNER(upload_raw(m, &d_both, both.data(), 2 * bytes));
-    RC_INNER(upload(m, &m->conv_sw[i], isw));
     ConvF32TcSpec sp{};
-    sp.x = m->qbuf;
-    sp.max_poses = m->d.max_poses;
+    // before the parts buffer exists the grid's address stands in for it (conv_f32tc_plan then tells whether a tile fits)
+    sp.x = m->qbuf ? m->qbuf : m->grid;
+    sp.max_poses = m->f32_parts;
     sp.n_in = m->conv[i].n_in;
-    sp.cin_pad = cp;
-    sp.w_hi = d_hi;
-    sp.w_both = d_both;
+    sp.cin_pad = f32tc_channels(m, i);
+    sp.w_hi = m->conv[i].w_hi;
+    sp.w_both = m->conv[i].w_both;
     sp.inv_sw = m->conv_sw[i];
     sp.inv_sx = m->qscale;
-    sp.bias = bias;
+    sp.bias = m->conv[i].b;
     sp.xres = i > 0 ? static_cast<const float *>(m->act[i - 1]) : nullptr;
     sp.y = static_cast<float *>(m->act[i]);
     sp.n_out = m->conv[i].n_out;
@@ -484,10 +474,53 @@ int plan_f32tc(fusion_model *m, int i, const float *w, float *bias) {
     sp.stride = c.stride;
     sp.residual = c.residual;
     sp.err = m->err;
-    sp.fold = fold;
+    sp.fold = i == 0 && m->f32_fold >= 0 ? 1 : 0;
     sp.blocked = f32tc_layout(m, i);
+    return sp;
+}
+
+// Whether FP32 layer i runs on the tensor cores, into m->f32tc[i], and its plan; a layer that no tile fits stays on the
+// CUDA cores.  FUSION_ENOMEM where the device refuses a plan (fusion_create then takes the CUDA cores for every layer).
+int plan_f32tc(fusion_model *m, int i) {
     char why[256] = {0};
-    m->f32tc[i] = conv_f32tc_plan(m->f32plan[i], sp, why, sizeof(why)) == 0;
+    const int r = m->f32_parts > 0 && conv_f32tc_block(m->d.conv[i].c_out)
+                      ? conv_f32tc_plan(m->f32plan[i], f32tc_spec(m, i), why, sizeof(why)) : -1;
+    if (r < -1) return fail(FUSION_ENOMEM, std::string("conv layer ") + std::to_string(i) + ": " + why);
+    m->f32tc[i] = r == 0;
+    return FUSION_OK;
+}
+
+int upload_f32tc_weights(fusion_model *m, int i, const float *w) {
+    const fusion_conv_desc &c = m->d.conv[i];
+    const ConvF32TcSpec sp = f32tc_spec(m, i);
+    const int nt = conv_f32tc_block(c.c_out);
+    const size_t bytes = conv_tc_weight_bytes(sp.cin_pad, nt, c.k, c.stride, 2, sp.fold) * (c.c_out / nt);
+    std::vector<uint8_t> hi(bytes), both(2 * bytes);
+    std::vector<float> isw(c.c_out);
+    conv_f32tc_arrange_weights(w, c.c_out, c.c_in, sp.cin_pad, c.k, c.stride, sp.fold, hi.data(), both.data(), isw.data());
+    RC_INNER(upload_raw(m, &m->conv[i].w_hi, hi.data(), bytes));
+    RC_INNER(upload_raw(m, &m->conv[i].w_both, both.data(), 2 * bytes));
+    return upload(m, &m->conv_sw[i], isw);
+}
+
+// The parts buffer, after everything else of the model: at most `limit` bytes (one pose at least), fewer poses where the
+// device has less, and the plans that read it.  A call of more poses takes each layer in several launches, with the same
+// results: full-size model, 18 poses to a launch (a launch is 26 rounds of tiles, the last one 0.6 full).
+int alloc_f32tc_parts(fusion_model *m, size_t limit) {
+    size_t pose = 0;
+    for (int i = 0; i < m->d.n_conv; ++i) {
+        const size_t n = m->conv[i].n_in;
+        if (m->f32tc[i]) pose = std::max(pose, n * n * n * f32tc_channels(m, i) * 4);
+    }
+    if (!pose) return FUSION_OK;
+    int rc = FUSION_ENOMEM;
+    for (int p = (int)std::min((size_t)m->d.max_poses, std::max(limit / pose, (size_t)1)); p > 0 && rc; p /= 2) {
+        rc = dalloc_bytes(m, &m->qbuf, p * pose);
+        m->f32_parts = p;
+    }
+    if (rc) return rc;
+    for (int i = 0; i < m->d.n_conv; ++i)
+        if (m->f32tc[i]) RC_INNER(plan_f32tc(m, i));
     return FUSION_OK;
 }
 
@@ -524,7 +557,8 @@ int load_weights(fusion_model *m, const float *blob) {
         }
         RC(upload(m, &m->conv[i].b, std::vector<float>(b, b + c.c_out)));
         m->conv[i].cx_in = cx;
-        if (!m->bf16) RC(plan_f32tc(m, i, w, m->conv[i].b));
+        if (!m->bf16) RC(plan_f32tc(m, i));
+        if (m->f32tc[i]) RC(upload_f32tc_weights(m, i, w));
         if (!m->bf16 && !m->f32tc[i]) {
             std::vector<float> t((size_t)k3 * cx * c.c_out, 0.f);
             for (int o = 0; o < c.c_out; ++o)
@@ -694,15 +728,8 @@ int alloc_workspace(fusion_model *m) {
         RC(dalloc(m, &m->qscale, B));
     }
     if (!m->bf16) {
-        // the largest layer input as two FP16 parts; without room for it the layers stay on the CUDA cores
-        size_t parts = 0;
-        for (int i = 0; i < d.n_conv; ++i) {
-            const size_t n = conv_out(d, i).n;
-            parts = std::max(parts, B * n * n * n * f32tc_channels(m, i) * 4);
-        }
         RC(dalloc(m, &m->amax, B));
         RC(dalloc(m, &m->qscale, B));
-        if (dalloc_bytes(m, &m->qbuf, parts) != FUSION_OK) m->qbuf = nullptr;
     }
     if (m->bf16) m->dense_tc_splits = dense_tc_splits(m->flat, d.cnn_dense);
     RC(dalloc(m, &m->dense_part, std::max((size_t)std::max(m->splits, m->dense_tc_splits) * B * d.cnn_dense,
@@ -918,6 +945,17 @@ void fusion_destroy(fusion_model *m) {
 int fusion_create(const fusion_model_desc *desc, const void *weights, size_t weights_bytes, void *cuda_stream,
                   fusion_model **out) {
     if (!out) return fail(FUSION_EINVAL, "out is NULL");
+    int rc = create_model(desc, weights, weights_bytes, cuda_stream, kF32PartsBytes, out);
+    // what an FP32 model on the tensor cores needs beyond the CUDA cores' must not refuse the model
+    if (rc == FUSION_ENOMEM && desc->dtype == FUSION_F32)
+        rc = create_model(desc, weights, weights_bytes, cuda_stream, 0, out);
+    return rc;
+}
+
+}  // extern "C"
+
+int fusion::create_model(const fusion_model_desc *desc, const void *weights, size_t weights_bytes, void *cuda_stream,
+                         size_t f32_parts_bytes, fusion_model **out) {
     std::string why;
     if (!check_desc(desc, &why)) return fail(FUSION_EINVAL, why);
 
@@ -950,6 +988,7 @@ int fusion_create(const fusion_model_desc *desc, const void *weights, size_t wei
     m->flat = f.c * f.n * f.n * f.n;
     m->splits = dense_splits(m->flat);
     m->bf16 = (m->d.dtype == FUSION_BF16 || m->d.dtype == FUSION_FP8);
+    m->f32_parts = !m->bf16 && f32_parts_bytes ? m->d.max_poses : 0;
     m->fp8 = (m->d.dtype == FUSION_FP8);
     m->sg_tc = m->bf16;
     m->sg_npw = default_npw(m);
@@ -972,6 +1011,7 @@ int fusion_create(const fusion_model_desc *desc, const void *weights, size_t wei
     }
     int rc = alloc_workspace(m);
     if (!rc) rc = load_weights(m, static_cast<const float *>(weights));
+    if (!rc) rc = alloc_f32tc_parts(m, f32_parts_bytes);
     if (!rc && m->bf16) rc = plan_tensor_core_convs(m);
     if (!rc && m->bf16) rc = plan_tensor_core_dense(m);
     if (!rc) sg_gru_tc_prepare(m->d.sg_hidden);
@@ -984,6 +1024,8 @@ int fusion_create(const fusion_model_desc *desc, const void *weights, size_t wei
     *out = m;
     return FUSION_OK;
 }
+
+extern "C" {
 
 static int check_launch(const char *what) {
     cudaError_t e = cudaGetLastError();
@@ -1190,13 +1232,16 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                 CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
                 launch_amax_f32(static_cast<const float *>(x), B, n * n * n * m->conv[i].cx_in, m->amax, st);
             }
-            SplitF16Args sa{static_cast<const float *>(x), static_cast<__half *>(m->qbuf), (int)n, m->conv[i].cx_in,
-                            f32tc_channels(m, i), d.max_poses, f32tc_layout(m, i), i == 0 ? m->f32_fold : -1, m->amax,
-                            m->qscale};
-            launch_split_f16(sa, B, st);
             const bool next = i + 1 < d.n_conv && m->f32tc[i + 1];
-            if (next) CU(cudaMemsetAsync(m->amax, 0, sizeof(float) * B, st));
-            m->last_tile[i] = conv_f32tc_launch(m->f32plan[i], B, next ? m->amax : nullptr, st);
+            for (int p0 = 0; p0 < B; p0 += m->f32_parts) {      // as many poses as the parts buffer holds
+                const int np = std::min(m->f32_parts, B - p0);
+                SplitF16Args sa{static_cast<const float *>(x) + p0 * n * n * n * m->conv[i].cx_in,
+                                static_cast<__half *>(m->qbuf), (int)n, m->conv[i].cx_in, f32tc_channels(m, i),
+                                m->f32_parts, f32tc_layout(m, i), i == 0 ? m->f32_fold : -1, m->amax + p0, m->qscale + p0};
+                launch_split_f16(sa, np, st);
+                if (next) CU(cudaMemsetAsync(m->amax + p0, 0, sizeof(float) * np, st));
+                m->last_tile[i] = conv_f32tc_launch(m->f32plan[i], p0, np, next ? m->amax + p0 : nullptr, st);
+            }
         } else {
             ConvArgs ca{static_cast<const float *>(x), static_cast<const float *>(m->conv[i].w), m->conv[i].b,
                         static_cast<float *>(m->act[i]), B, m->conv[i].n_in, m->conv[i].n_out,

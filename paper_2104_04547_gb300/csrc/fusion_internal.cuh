@@ -241,22 +241,23 @@ struct ConvF32TcPlan {
 };
 struct ConvF32TcSpec {
     const void *x;          // the input's FP16 parts (launch_split_f16): [2][max_poses] maps of cin_pad channels
-    int max_poses, n_in, cin_pad;
+    int max_poses, n_in, cin_pad;   // poses a launch takes at most
     const void *w_hi, *w_both;   // arranged weights (conv_f32tc_arrange_weights)
     const float *inv_sw;    // [c_out] 1 / weight scale
-    const float *inv_sx;    // [max_poses] 1 / input scale
+    const float *inv_sx;    // [poses of the call] 1 / input scale
     const float *bias;      // [c_out]
-    const float *xres;      // residual source [max_poses][n_in]^3[c_out]
-    float *y;               // [max_poses][n_out]^3[c_out], NDHWC
+    const float *xres;      // residual source [poses of the call][n_in]^3[c_out]
+    float *y;               // [poses of the call][n_out]^3[c_out], NDHWC
     int n_out, c_out, k, stride, residual;
     unsigned *err;
     int fold;               // 1: x-folded first-layer input (launch_split_f16 with fold_pad = k / 2)
     int blocked;            // layout of the parts: 0 NDHWC, 1 channel-blocked, 2 parity-split (ConvTcSpec::blocked)
 };
-// 0, or nonzero with a reason: the caller then uses launch_conv3d_f32.
+// 0; -1 with a reason where no tile fits (the caller then uses launch_conv3d_f32); -2 where the device refused.
 int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &spec, char *why, size_t why_len);
-// amax: per-pose max |output| (atomic max, zeroed by the caller), or null.  Returns the tile.
-ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s);
+// Poses p0 .. p0 + B - 1 of the call, whose parts are the buffer's poses 0 .. B - 1.  amax: their max |output| (atomic max,
+// zeroed by the caller), or null.  Returns the tile.
+ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s);
 // Output channels per tile (0: c_out is not a multiple of 32).
 int conv_f32tc_block(int c_out);
 // Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two; inv_sw[co] = 1 / s_w[co].  Per block of
@@ -433,5 +434,11 @@ void launch_head(const HeadArgs &a, cudaStream_t s);
 
 // Record `msg` as the calling thread's fusion_last_error() message; returns `code`.
 int set_last_error(int code, const char *msg);
+
+// fusion_create with a limit on the FP16 parts buffer of an FP32 model: f32_parts_bytes (one pose's at least), 0 = its
+// convolutions on the CUDA cores.  Scores are the same for every limit but 0; no other limit is taken in its place.
+constexpr size_t kF32PartsBytes = (size_t)512 << 20;
+int create_model(const fusion_model_desc *desc, const void *weights, size_t weights_bytes, void *cuda_stream,
+                 size_t f32_parts_bytes, fusion_model **out);
 
 }  // namespace fusion

@@ -76,7 +76,7 @@ struct Args {
     const uint8_t *w[2];   // arranged weights (conv_f32tc_arrange_weights): w_hi, and [w_hi | w_lo]
     size_t wblk;           // bytes of w[0] per block of NT output channels
     const float *inv_sw;   // [c_out] 1 / s_w
-    const float *inv_sx;   // [B] 1 / s_x
+    const float *inv_sx;   // [B] 1 / s_x (this and the maps below from the launch's first pose on)
     const float *bias;     // [c_out]
     const float *xres;     // residual source [B][n_out]^3[c_out], or unused
     float *y;              // [B][n_out]^3[c_out]
@@ -762,7 +762,7 @@ static void launch_t(const ConvF32TcPlan::Impl &P, const ConvF32TcPlan::Impl::Va
     conv3d_f32tc_kernel<NT, T><<<grid, Roles<NT, T>::THREADS, V.smem, s>>>(V.tmap, a);
 }
 
-ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaStream_t s) {
+ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s) {
     const ConvF32TcPlan::Impl &P = *plan.impl;
     // the tile with the shortest schedule: rounds of tiles over the SMs x a tile's MMA clocks
     int best = 0;
@@ -778,6 +778,11 @@ ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int B, float *amax, cudaSt
     a.g = V.g;
     a.B = B;
     a.amax = amax;
+    // an output map has n_out^3 c_out floats, and so has a residual source (stride 1, c_in = c_out)
+    const size_t maps = (size_t)p0 * a.n_out * a.n_out * a.n_out * a.c_out;
+    a.inv_sx += p0;
+    a.y += maps;
+    if (a.residual) a.xres += maps;
     switch (P.NT * 16 + V.T) {
     case 32 * 16 + 8: launch_t<32, 8>(P, V, a, s); break;
     case 32 * 16 + 4: launch_t<32, 4>(P, V, a, s); break;

@@ -150,6 +150,80 @@ void worker_loop(fusion_server *s, int si) {
 
 int srv_fail(int code, const std::string &m) { return fusion::set_last_error(code, m.c_str()); }
 
+void close_slots(fusion_server *s) {
+    for (auto &sl : s->slots) {
+        fusion_destroy(sl.model);
+        cudaFreeHost(sl.off);
+        cudaFreeHost(sl.nlig);
+        cudaFreeHost(sl.xyz);
+        cudaFreeHost(sl.feat);
+        cudaFreeHost(sl.out);
+    }
+    s->slots.clear();
+}
+
+// The server's slots, FP32 ones with at most f32_parts bytes of parts buffer.  *all: every slot asked for was admitted.
+// On failure (a dtype without a slot) the slots made so far stay, for close_slots.
+int open_slots(fusion_server *s, const fusion_model_desc *desc, const void *weights, size_t weights_bytes, size_t f32_parts,
+               bool *all) {
+    const fusion_server_config &cfg = s->cfg;
+    s->slot_bytes = 0;
+    int dts[kDtypes], ndt = 0;
+    for (int t = 0; t < kDtypes; ++t)
+        if (s->dtype_mask & (1u << t)) dts[ndt++] = t;
+    fusion_model_desc d = *desc;
+    d.max_poses = cfg.max_batch;
+    const int want = std::max(cfg.slots > 0 ? cfg.slots : 4, ndt);
+    size_t used = 0;
+    for (int i = 0; i < want; ++i) {
+        // slots cycle through the dtypes; HBM budget admission: a further slot is created only if all slots
+        // fit the budget (a dtype's footprint is measured on its first slot)
+        const int dt = dts[i % ndt];
+        const bool first_of_dtype = i < ndt;
+        if (cfg.hbm_budget_bytes > 0 && !first_of_dtype && used + s->dtype_bytes[dt] > cfg.hbm_budget_bytes) break;
+        size_t free0 = 0, free1 = 0, total = 0;
+        cudaMemGetInfo(&free0, &total);
+        Slot sl;
+        sl.dtype = dt;
+        d.dtype = dt;
+        int rc = fusion::create_model(&d, weights, weights_bytes, nullptr, f32_parts, &sl.model);
+        if (rc) {
+            if (first_of_dtype) return rc;
+            break;   // no memory for more slots: serve with the ones admitted
+        }
+        cudaMemGetInfo(&free1, &total);
+        if (first_of_dtype) {
+            s->dtype_bytes[dt] = free0 > free1 ? free0 - free1 : 0;
+            s->slot_bytes = std::max(s->slot_bytes, s->dtype_bytes[dt]);
+            if (cfg.hbm_budget_bytes > 0 && used + s->dtype_bytes[dt] > cfg.hbm_budget_bytes) {
+                const size_t need = s->dtype_bytes[dt];
+                fusion_destroy(sl.model);
+                return srv_fail(FUSION_ENOMEM, "one slot (" + std::to_string(need) + " bytes) exceeds the HBM budget");
+            }
+        }
+        used += s->dtype_bytes[dt];
+        const size_t A = (size_t)cfg.max_batch * desc->max_atoms;
+        if (cudaMallocHost(&sl.off, sizeof(int32_t) * (cfg.max_batch + 1)) != cudaSuccess ||
+            cudaMallocHost(&sl.nlig, sizeof(int32_t) * cfg.max_batch) != cudaSuccess ||
+            cudaMallocHost(&sl.xyz, sizeof(float) * A * 3) != cudaSuccess ||
+            cudaMallocHost(&sl.feat, sizeof(float) * A * 19) != cudaSuccess ||
+            cudaMallocHost(&sl.out, sizeof(float) * cfg.max_batch) != cudaSuccess) {
+            fusion_destroy(sl.model);
+            cudaFreeHost(sl.off);
+            cudaFreeHost(sl.nlig);
+            cudaFreeHost(sl.xyz);
+            cudaFreeHost(sl.feat);
+            cudaFreeHost(sl.out);
+            cudaGetLastError();
+            if (first_of_dtype) return srv_fail(FUSION_ENOMEM, "pinned host buffers for a slot");
+            break;
+        }
+        s->slots.push_back(sl);
+    }
+    *all = (int)s->slots.size() == want;
+    return FUSION_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -169,65 +243,21 @@ int fusion_server_create(const fusion_model_desc *desc, const void *weights, siz
     s->max_atoms = desc->max_atoms;
     s->default_dtype = desc->dtype;
     s->dtype_mask = (unsigned)cfg->dtypes | (1u << desc->dtype);
-    int dts[kDtypes], ndt = 0;
-    for (int t = 0; t < kDtypes; ++t)
-        if (s->dtype_mask & (1u << t)) dts[ndt++] = t;
     cudaGetDevice(&s->device);
-    fusion_model_desc d = *desc;
-    d.max_poses = cfg->max_batch;
-    const int want = std::max(cfg->slots > 0 ? cfg->slots : 4, ndt);
-    size_t used = 0;
-    for (int i = 0; i < want; ++i) {
-        // slots cycle through the dtypes; HBM budget admission: a further slot is created only if all slots
-        // fit the budget (a dtype's footprint is measured on its first slot)
-        const int dt = dts[i % ndt];
-        const bool first_of_dtype = i < ndt;
-        if (cfg->hbm_budget_bytes > 0 && !first_of_dtype && used + s->dtype_bytes[dt] > cfg->hbm_budget_bytes) break;
-        size_t free0 = 0, free1 = 0, total = 0;
-        cudaMemGetInfo(&free0, &total);
-        Slot sl;
-        sl.dtype = dt;
-        d.dtype = dt;
-        int rc = fusion_create(&d, weights, weights_bytes, nullptr, &sl.model);
-        if (rc) {
-            if (first_of_dtype) {
-                fusion_server_destroy(s);
-                return rc;
-            }
-            break;   // no memory for more slots: serve with the ones admitted
+    // The parts buffer of FP32 slots (kF32PartsBytes) gives way where the device or the budget is short: to a sixteenth of a
+    // slot when not every slot was admitted, to one pose and then to none (convolutions on the CUDA cores) when a dtype
+    // got no slot.  All slots take the same limit, so that a pose's score does not depend on its slot.
+    size_t parts = fusion::kF32PartsBytes;
+    for (;;) {
+        bool all = false;
+        const int rc = open_slots(s, desc, weights, weights_bytes, parts, &all);
+        if (rc == FUSION_OK && (all || parts != fusion::kF32PartsBytes || !(s->dtype_mask & (1u << FUSION_F32)))) break;
+        if (rc && (rc != FUSION_ENOMEM || parts == 0 || !(s->dtype_mask & (1u << FUSION_F32)))) {
+            fusion_server_destroy(s);               // (keeps the message of the failure)
+            return rc;
         }
-        cudaMemGetInfo(&free1, &total);
-        if (first_of_dtype) {
-            s->dtype_bytes[dt] = free0 > free1 ? free0 - free1 : 0;
-            s->slot_bytes = std::max(s->slot_bytes, s->dtype_bytes[dt]);
-            if (cfg->hbm_budget_bytes > 0 && used + s->dtype_bytes[dt] > cfg->hbm_budget_bytes) {
-                const size_t need = s->dtype_bytes[dt];
-                fusion_destroy(sl.model);
-                fusion_server_destroy(s);
-                return srv_fail(FUSION_ENOMEM, "one slot (" + std::to_string(need) + " bytes) exceeds the HBM budget");
-            }
-        }
-        used += s->dtype_bytes[dt];
-        const size_t A = (size_t)cfg->max_batch * desc->max_atoms;
-        if (cudaMallocHost(&sl.off, sizeof(int32_t) * (cfg->max_batch + 1)) != cudaSuccess ||
-            cudaMallocHost(&sl.nlig, sizeof(int32_t) * cfg->max_batch) != cudaSuccess ||
-            cudaMallocHost(&sl.xyz, sizeof(float) * A * 3) != cudaSuccess ||
-            cudaMallocHost(&sl.feat, sizeof(float) * A * 19) != cudaSuccess ||
-            cudaMallocHost(&sl.out, sizeof(float) * cfg->max_batch) != cudaSuccess) {
-            fusion_destroy(sl.model);
-            cudaFreeHost(sl.off);
-            cudaFreeHost(sl.nlig);
-            cudaFreeHost(sl.xyz);
-            cudaFreeHost(sl.feat);
-            cudaFreeHost(sl.out);
-            cudaGetLastError();
-            if (first_of_dtype) {
-                fusion_server_destroy(s);
-                return srv_fail(FUSION_ENOMEM, "pinned host buffers for a slot");
-            }
-            break;
-        }
-        s->slots.push_back(sl);
+        parts = rc ? (parts > 1 ? 1 : 0) : std::max(s->dtype_bytes[FUSION_F32] / 16, (size_t)1);
+        close_slots(s);
     }
     for (int i = 0; i < (int)s->slots.size(); ++i) s->workers.emplace_back(worker_loop, s, i);
     *out = s;
@@ -325,14 +355,7 @@ void fusion_server_destroy(fusion_server *s) {
     }
     for (auto &cv : s->cv_work) cv.notify_all();
     for (auto &t : s->workers) t.join();
-    for (auto &sl : s->slots) {
-        fusion_destroy(sl.model);
-        cudaFreeHost(sl.off);
-        cudaFreeHost(sl.nlig);
-        cudaFreeHost(sl.xyz);
-        cudaFreeHost(sl.feat);
-        cudaFreeHost(sl.out);
-    }
+    close_slots(s);
     delete s;
 }
 

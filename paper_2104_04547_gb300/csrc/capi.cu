@@ -1233,10 +1233,8 @@ static int enqueue_forward(fusion_model *m, int B, int A, int most_atoms, const 
                 launch_amax_f32(static_cast<const float *>(x), B, n * n * n * m->conv[i].cx_in, m->amax, st);
             }
             const bool next = i + 1 < d.n_conv && m->f32tc[i + 1];
-            // launches of equal numbers of poses, as many as the parts buffer makes necessary
-            const int launches = (B + m->f32_parts - 1) / m->f32_parts, each = (B + launches - 1) / launches;
-            for (int p0 = 0; p0 < B; p0 += each) {
-                const int np = std::min(each, B - p0);
+            for (int p0 = 0; p0 < B; p0 += m->f32_parts) {      // as many poses as the parts buffer holds
+                const int np = std::min(m->f32_parts, B - p0);
                 SplitF16Args sa{static_cast<const float *>(x) + p0 * n * n * n * m->conv[i].cx_in,
                                 static_cast<__half *>(m->qbuf), (int)n, m->conv[i].cx_in, f32tc_channels(m, i),
                                 m->f32_parts, f32tc_layout(m, i), i == 0 ? m->f32_fold : -1, m->amax + p0, m->qscale + p0};

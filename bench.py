@@ -42,21 +42,21 @@ L2_FLUSH_BYTES = 256 << 20
 # tensor but the weights scales with the pose count).  Valid only for the kernel source they were taken
 # on: the sha256 prefix of the conv kernel's source code (comments removed); other code reports null.
 CONV_TRAFFIC = {
-    "src": "4a85110ed9c3a3cd",
+    "src": "a86df3d04d93fbee",
     "poses": 64,
-    "bf16": [1130.8e6, 1665.9e6, 1681.7e6, 1052.2e6],
-    "fp8": [1149.3e6, 2100.8e6, 2103.2e6, 555.7e6],
+    "bf16": [1127.2e6, 1668.3e6, 1671.8e6, 1052.3e6],
+    "fp8": [1149.3e6, 2101.2e6, 2105.1e6, 558.1e6],
 }
 
 
 # DRAM bytes of one voxelize launch at 64 poses (ncu dram__bytes_read.sum + dram__bytes_write.sum), valid for the
 # voxelize source they were taken on (sha256 prefix as for the conv); otherwise null.
-# Taken on 32 poses (171.50 MB = 3.46 MB read + 168.04 MB written) and scaled x2: the grid and the records scale
+# Taken on 32 poses (171.63 MB = 3.49 MB read + 168.13 MB written) and scaled x2: the grid and the records scale
 # with the pose count.  Part of a launch's writes can still sit in L2 when it ends, so this undercounts slightly.
 VOX_TRAFFIC = {
-    "src": "78415aeadf2a5dbd",
+    "src": "25a8304cd6c91ebf",
     "poses": 64,
-    "bf16": 2 * 171.50e6,
+    "bf16": 2 * 171.63e6,
 }
 
 

@@ -47,6 +47,12 @@ inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// |v|, or 0 where v is infinite or NaN: the scale of an FP32 map's FP16 parts is that of its finite values.
+__device__ __forceinline__ float finite_abs(float v) {
+    const float a = fabsf(v);
+    return a < INFINITY ? a : 0.f;
+}
+
 constexpr int kFeat = 19;
 constexpr int kMaxSupportW = 11;     // 2k+1 for k <= 5
 constexpr int kGridCellsMax = 16;    // graph cell list: at most 16 cells per axis
@@ -96,7 +102,8 @@ struct VoxArgs {
     int blocked;          // bf16 only: store channel-blocked, [B][n][n][cx / 8][n][8]
     const int32_t *cell_row;     // PrepArgs::cell_row
     const float *atom_rec;       // PrepArgs::atom_rec (records in cell order)
-    float *amax;          // cx 24 or 32, may be null: per-pose max |stored value| (atomic max; zeroed by the caller)
+    float *amax;          // cx 24 or 32, may be null: per-pose max |stored value| (float32: of the finite ones; atomic max,
+                          // zeroed by the caller)
 };
 void launch_voxelize(const VoxArgs &a, cudaStream_t s);
 
@@ -255,12 +262,13 @@ struct ConvF32TcSpec {
 };
 // 0; -1 with a reason where no tile fits (the caller then uses launch_conv3d_f32); -2 where the device refused.
 int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &spec, char *why, size_t why_len);
-// Poses p0 .. p0 + B - 1 of the call, whose parts are the buffer's poses 0 .. B - 1.  amax: their max |output| (atomic max,
-// zeroed by the caller), or null.  Returns the tile.
+// Poses p0 .. p0 + B - 1 of the call, whose parts are the buffer's poses 0 .. B - 1.  amax: their max |output|, infinities
+// aside (atomic max, zeroed by the caller), or null.  Returns the tile.
 ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s);
 // Output channels per tile (0: c_out is not a multiple of 32).
 int conv_f32tc_block(int c_out);
-// Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two; inv_sw[co] = 1 / s_w[co].  Per block of
+// Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two (of the channel's finite weights; an infinite
+// or NaN weight is hi = itself, lo = 0); inv_sw[co] = 1 / s_w[co].  Per block of
 // NT = conv_f32tc_block(c_out) output channels, in the layout of conv_tc_arrange_weights (elem 2) for NT channels:
 // w_hi has rows [tz][hi of NT channels], w_both rows [tz][hi of NT channels, lo of NT channels].  w_hi takes
 // c_out / NT x conv_tc_weight_bytes(cin_pad, NT, k, stride, 2, fold) bytes, w_both twice that.
@@ -273,11 +281,11 @@ struct SplitF16Args {
     int n, c, cp, max_poses;
     int layout;             // 0 NDHWC, 1 channel-blocked, 2 parity-split
     int fold_pad;           // >= 0 (cp = 32, layout 1): channels 16..18 folded along x as in VoxArgs::fold_pad
-    const float *amax;      // [B] max |x| of each pose
+    const float *amax;      // [B] max |x| of each pose, infinities and NaN aside
     float *inv_sx;          // [B] 2^-e
 };
 void launch_split_f16(const SplitF16Args &a, int B, cudaStream_t s);
-// Per-pose max |x| of FP32 maps (atomic max, zeroed by the caller); per_pose a multiple of 4.
+// Per-pose max |x| of FP32 maps, infinities and NaN aside (atomic max, zeroed by the caller); per_pose a multiple of 4.
 void launch_amax_f32(const float *x, int B, size_t per_pose, float *amax, cudaStream_t s);
 
 // Per-pose FP8 quantization of the channel-blocked bf16 grid [B][n][n][3][n][8] (channels 0..18) into the folded layout

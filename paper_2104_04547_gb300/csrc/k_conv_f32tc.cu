@@ -15,6 +15,12 @@
 // FP32 with rounding, to the outputs' totals in their registers.  Intervals and the order of every sum depend on the
 // layer only (not on the tile or the batch), so a pose's result depends on nothing but the pose.
 //
+// Infinities and NaN: the scales are those of the finite values, an infinity's low part is 0 and sums of small products
+// that are not finite are left out, so that x_hi w_hi alone gives an output what a chain of multiply-adds would: the
+// infinity of its sign, NaN where two disagree, and every output whose terms are finite keeps its value.  (In a folded
+// 7^3 first layer an infinity of features 16..18 meets the zero weights of slots read twice: outputs within a voxel of it
+// along x are NaN, stored as 0.)
+//
 // Tiles: M = 128 voxels (16 x 8), T output slices and NT output channels per CTA.  Operand A is read from a
 // TMA-loaded halo by sliding descriptors as in k_conv_tc.cu, weights stream in whole (ty, tx) groups.  The
 // halo of x_lo is multiplied with w_hi (N = NT), the halo of x_hi with [w_hi | w_lo] (N = 2 NT), so one read of
@@ -417,12 +423,15 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
                         tc::tc_fence_after();
                         const uint32_t tu = tsub + (uint32_t)(s * UCOLS);
                         // 16 columns at a time: 32 more registers beside the totals would spill
-                        auto add16 = [&](int col, int c16) {
+                        auto add16 = [&](int col, int c16, bool finite_only) {
                             uint32_t v[16];
                             tc::tmem_ld16(tu + (uint32_t)(col + c16), v);
                             tc::tmem_ld_wait();
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) tot[o][c16 + j] += __uint_as_float(v[j]);
+                            for (int j = 0; j < 16; ++j) {
+                                const float t = __uint_as_float(v[j]);
+                                if (!finite_only || fabsf(t) < INFINITY) tot[o][c16 + j] += t;
+                            }
                         };
                         auto zero = [&](int col) {
 #pragma unroll
@@ -430,11 +439,11 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
                         };
                         if (i == per_tile - 1) {      // the tile's small products are complete
 #pragma unroll
-                            for (int c16 = 0; c16 < NT; c16 += 16) add16(NT, c16);
+                            for (int c16 = 0; c16 < NT; c16 += 16) add16(NT, c16, true);
                             zero(NT);
                         }
 #pragma unroll
-                        for (int c16 = 0; c16 < NT; c16 += 16) add16(0, c16);
+                        for (int c16 = 0; c16 < NT; c16 += 16) add16(0, c16, false);
                         zero(0);
                         tc::tmem_st_wait();
                         tc::tc_fence_before();
@@ -468,7 +477,7 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
                         const float4 x4 = __ldg(reinterpret_cast<const float4 *>(a.xres + at) + j4);
                         v.x += x4.x; v.y += x4.y; v.z += x4.z; v.w += x4.w;
                     }
-                    vmax = fmaxf(vmax, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+                    vmax = fmaxf(vmax, fmaxf(fmaxf(finite_abs(v.x), finite_abs(v.y)), fmaxf(finite_abs(v.z), finite_abs(v.w))));
                     reinterpret_cast<float4 *>(a.y + at)[j4] = v;
                 }
             }
@@ -544,11 +553,12 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitF16Args a) {
         const int x = (int)(v - row * n);
         float f[8];
         if (a.fold_pad >= 0 && cb >= 2) {
-            // x-folded second chunk: slot 3 s + c = channel 16 + c of voxel x - p + s (slot 15 unused)
+            // x-folded second chunk: slot 3 s + c = channel 16 + c of voxel x - p + s, s < k (slot 15 unused)
+            const int used = 3 * min(5, 2 * a.fold_pad + 1);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int sl = (cb - 2) * 8 + j, xs = x - a.fold_pad + sl / 3;
-                f[j] = sl < 15 && xs >= 0 && xs < n ? xb[(row * n + xs) * a.c + 16 + sl % 3] : 0.f;
+                f[j] = sl < used && xs >= 0 && xs < n ? xb[(row * n + xs) * a.c + 16 + sl % 3] : 0.f;
             }
         } else if (cb * 8 < a.c) {
             const float4 *src = reinterpret_cast<const float4 *>(xb + v * a.c + cb * 8);   // c is a multiple of 8
@@ -584,7 +594,7 @@ __global__ void __launch_bounds__(256) amax_f32_kernel(const float *x, size_t pe
     float m = 0.f;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < per_pose / 4; i += (size_t)gridDim.x * blockDim.x) {
         const float4 v = src[i];
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        m = fmaxf(m, fmaxf(fmaxf(finite_abs(v.x), finite_abs(v.y)), fmaxf(finite_abs(v.z), finite_abs(v.w))));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned *>(amax + b), __float_as_uint(m));

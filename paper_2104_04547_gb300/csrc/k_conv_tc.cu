@@ -924,10 +924,14 @@ void conv_f32tc_arrange_weights(const float *w, int c_out, int c_in, int cin_pad
     const int NT = conv_f32tc_block(c_out);
     std::vector<float> s(c_out);
     for (int co = 0; co < c_out; ++co) {
-        // 2^e puts the channel's largest weight in [2^14, 2^15)
-        const float mx = channel_max(w, co, per);
+        // 2^e puts the channel's largest finite weight in [2^14, 2^15)
+        float mx = 0.f;
+        for (size_t q = 0; q < per; ++q) {
+            const float v = std::fabs(w[(size_t)co * per + q]);
+            if (v > mx && std::isfinite(v)) mx = v;
+        }
         int e = 0;
-        if (mx > 0.f && std::isfinite(mx)) e = 14 - std::ilogb(mx);
+        if (mx > 0.f) e = 14 - std::ilogb(mx);
         if (e > 126) e = 126;
         s[co] = std::ldexp(1.f, e);
         inv_sw[co] = std::ldexp(1.f, -e);

@@ -437,7 +437,8 @@ __global__ void __launch_bounds__(kVoxThreads, 6) voxelize_kernel(VoxArgs a) {
                     v4.z = c0 + 2 < kFeat ? acc[c0 + 2 < kFeat ? c0 + 2 : 0] : 0.f;
                     v4.w = c0 + 3 < kFeat ? acc[c0 + 3 < kFeat ? c0 + 3 : 0] : 0.f;
                     *reinterpret_cast<float4 *>(out + c0) = v4;
-                    if (AMAX) vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(v4.x), fabsf(v4.y))), fmaxf(fabsf(v4.z), fabsf(v4.w)));
+                    if (AMAX) vmax = fmaxf(fmaxf(vmax, fmaxf(finite_abs(v4.x), finite_abs(v4.y))),
+                                           fmaxf(finite_abs(v4.z), finite_abs(v4.w)));
                 }
             }
         }

@@ -156,6 +156,10 @@ __device__ __forceinline__ void issue_nz(int nz, uint32_t on, uint32_t dt, uint3
     }
 }
 
+// t / (s_w s_x) from the inverse scales, powers of two from 2^-126 to 2^113: the smaller one first, so that no step
+// overflows, or goes below the normal range, where the result does not.
+__device__ __forceinline__ float unscale(float t, float isw, float isx) { return t * fminf(isw, isx) * fmaxf(isw, isx); }
+
 template <int NT, int T>
 __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                 Args a) {
@@ -469,10 +473,10 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
                     const float4 bs = __ldg(reinterpret_cast<const float4 *>(a.bias + c0) + j4);
                     const float *t = tot[o] + j4 * 4;
                     float4 v;
-                    v.x = fmaxf(t[0] * sw.x * isx + bs.x, 0.f);
-                    v.y = fmaxf(t[1] * sw.y * isx + bs.y, 0.f);
-                    v.z = fmaxf(t[2] * sw.z * isx + bs.z, 0.f);
-                    v.w = fmaxf(t[3] * sw.w * isx + bs.w, 0.f);
+                    v.x = fmaxf(unscale(t[0], sw.x, isx) + bs.x, 0.f);
+                    v.y = fmaxf(unscale(t[1], sw.y, isx) + bs.y, 0.f);
+                    v.z = fmaxf(unscale(t[2], sw.z, isx) + bs.z, 0.f);
+                    v.w = fmaxf(unscale(t[3], sw.w, isx) + bs.w, 0.f);
                     if (a.residual) {
                         const float4 x4 = __ldg(reinterpret_cast<const float4 *>(a.xres + at) + j4);
                         v.x += x4.x; v.y += x4.y; v.z += x4.z; v.w += x4.w;

@@ -76,3 +76,17 @@ def test_an_infinite_weight(F_):
     m.score(batch)
     found = _check_layers(F_, m, conv, W, n, 0)
     assert found[0] == 0 and found[1] > 0
+
+
+@pytest.mark.parametrize("w_exp,x_exp", [(115, -110), (-110, 100)])
+def test_scales_far_apart(F_, w_exp, x_exp):
+    """Weights and densities at opposite ends of FP32's range, whose products are ordinary numbers: no step overflows."""
+    n, conv = 14, [_cv(19, 64, 3), _cv(64, 32, 3, 2)]
+    desc = _desc(n, conv)
+    W = weights.init_weights(desc, 3)
+    W["conv0.w"] = W["conv0.w"] * np.float32(2.0 ** w_exp)
+    batch = poses.pack([poses.make_pose(101, (6, 8), (10, 20))])
+    batch["feat"] = batch["feat"] * np.float32(2.0 ** x_exp)
+    m = F_.Model(desc, weights.to_blob(desc, W), max_poses=1, max_atoms=64, keep_stages=True)
+    m.score(batch)
+    assert _check_layers(F_, m, conv, W, n, 0) == [0, 0]

@@ -15,9 +15,11 @@
 // further warp issues the MMAs: per 16 of K, w0 x0 (N = 64), w0 [x1 x2], w1 [x0 x1] (N = 128) and w2 x0 (N = 64).  Tensor memory:
 // columns [0, 384) the six sums of w0 x0, [384, 448) w0 x1 + w1 x0, [448, 512) the three smallest.
 //
-// Infinite, NaN or overflowing inputs make an output of the split form NaN where multiply-adds give an infinity, so an
-// output that is not finite is recomputed by a plain chain over the CTA's K range.  A bounded wait that runs out (none
-// should) does the same for every output.
+// Infinities and NaN: a first part is at most BF16's largest number, so that an infinity is its second part (its third is
+// NaN), a large finite value still the sum of its parts, and an output that uses them the infinity or NaN of a chain of
+// multiply-adds, once a sum of the smallest products that is not finite is left out.  (Recomputing such outputs by chains
+// instead took 4.1 ms for one infinite weight and 13.6 ms for NaN operands at 64 x 256 x 221,184.)  A bounded wait that
+// runs out (none should) has every output of the CTA computed by a plain chain over its K range.
 //
 // Bound: HBM and the latency of the copy - split - MMA chain: 64 x 256 x 221,184 takes 73 us (3.9 TB/s of the 283 MB; 266
 // us for the split-K kernel of the CUDA cores that was here, 197 us for its successor), 17 x 128 x 110,592 27 us.  Error
@@ -47,11 +49,13 @@ constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s
 
 __device__ __forceinline__ uint32_t pack(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t *>(&v); }
 
-// x -> bf16 parts p[0] + p[1] + p[2] of a pair of values.
+// x -> bf16 parts p[0] + p[1] + p[2] of a pair of values, |p[0]| at most BF16's largest number.
 __device__ __forceinline__ void split3(float a, float b, uint32_t (&p)[3]) {
+    const __nv_bfloat16 top = __ushort_as_bfloat16(0x7F7F), bottom = __ushort_as_bfloat16(0xFF7F);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        if (i == 0) h = __hmax2(__hmin2(h, __nv_bfloat162(top, top)), __nv_bfloat162(bottom, bottom));
         p[i] = pack(h);
         a -= __uint_as_float(p[i] << 16);
         b -= __uint_as_float(p[i] & 0xffff0000u);
@@ -191,14 +195,17 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
         float tot[kN];
 #pragma unroll
         for (int j = 0; j < kN; ++j) tot[j] = 0.f;
-        auto add = [&](int col) {
+        auto add = [&](int col, bool finite_only) {
 #pragma unroll
             for (int c = 0; c < kN; c += 16) {       // 16 at a time: 32 registers beside the totals would spill
                 uint32_t v[16];
                 tc::tmem_ld16(tbase + lanes + (uint32_t)(col + c), v);
                 tc::tmem_ld_wait();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) tot[c + j] += __uint_as_float(v[j]);
+                for (int j = 0; j < 16; ++j) {
+                    const float t = __uint_as_float(v[j]);
+                    if (!finite_only || fabsf(t) < INFINITY) tot[c + j] += t;
+                }
             }
         };
         bool ok = true;
@@ -209,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
                  !__any_sync(0xffffffffu, *failed != 0);
             if (!ok) break;
             tc::tc_fence_after();
-            add(acc * kN);
+            add(acc * kN, false);
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&sum_empty[acc]);
@@ -217,8 +224,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
         ok = __all_sync(0xffffffffu, ok && tc::mbar_wait(done, 0, deadline)) && !__any_sync(0xffffffffu, *failed != 0);
         if (ok) {
             tc::tc_fence_after();
-            add((kSums + 1) * kN);
-            add(kSums * kN);
+            add((kSums + 1) * kN, true);
+            add(kSums * kN, false);
         } else {
             *failed = 1;
         }
@@ -228,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
                 const int b = b0 + j;
                 if (b >= a.B) break;
                 float s = tot[j];
-                if (!ok || !isfinite(s)) {
+                if (!ok) {
                     const float *w = a.w + (size_t)n * a.K, *x = a.x + (size_t)b * a.K;
                     s = 0.f;
                     for (int k = kbeg; k < kend; ++k) s = fmaf(x[k], w[k], s);

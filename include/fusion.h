@@ -382,9 +382,11 @@ void fusion_server_destroy(fusion_server *s);
  *
  * y[b][n] = act(bias[n] + sum_k x[b][k] * w[n][k]) for b < B, n < N (act =
  * ReLU when relu != 0, identity otherwise): the CNN dense layer of
- * fusion_score in FP32, run as split-K kernels (more than 8 rows on the tensor
- * cores, each operand in three BF16 parts: FP32's accuracy, and sums whose
- * order depends on B), for callers that cannot allocate device memory.  Such callers include a serving process that admits
+ * fusion_score in FP32, run as split-K kernels, for callers that cannot
+ * allocate device memory.  Up to 8 rows take fusion_score's kernels and give
+ * its bits; more rows take the tensor cores, each operand in three BF16 parts
+ * (FP32's accuracy, sums in another order).  Within either range a row's bits
+ * do not depend on the other rows or their number.  Such callers include a serving process that admits
  * requests against a device-memory budget it does not own, a host application
  * whose own allocator owns every byte of the device, and a latency-bound
  * request loop that cannot take the implicit synchronisation and unbounded

@@ -137,9 +137,9 @@ struct DenseArgs {
     bool early;           // see launch_kernel
 };
 void launch_dense(const DenseArgs &a, cudaStream_t s);
-// The same layer on the tensor cores at FP32's accuracy (k_dense_f32tc.cu), with at most a.splits splits; the order of
-// additions depends on the batch.
-void launch_dense_f32tc(DenseArgs a, cudaStream_t s);
+// The same layer on the tensor cores at FP32's accuracy (k_dense_f32tc.cu), its split of K a function of N, K and the
+// device's `sms` multiprocessors (not of the batch, nor a.splits).  a.part: `partials` floats, 128 sms and N at least.
+void launch_dense_f32tc(DenseArgs a, size_t partials, int sms, cudaStream_t s);
 int dense_splits(int K);
 // The fixed-order split reduction + bias + activation of launch_dense, on partials [splits][B][N].
 void launch_dense_reduce(const DenseArgs &a, cudaStream_t s);

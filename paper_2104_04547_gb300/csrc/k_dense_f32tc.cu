@@ -251,15 +251,26 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
 
 }  // namespace
 
-void launch_dense_f32tc(DenseArgs a, cudaStream_t s) {
-    // about one CTA per SM, at most a.splits (the partials' room) and no fewer than 512 of K each, in whole stages
-    const int mt = (a.N + kM - 1) / kM, bt = (a.B + kN - 1) / kN;
-    const int want = std::max(1, std::min({a.splits, 152 / (mt * bt), (a.K + 511) / 512}));
+void launch_dense_f32tc(DenseArgs a, size_t partials, int sms, cudaStream_t s) {
+    // about one CTA per SM for 64 rows, no fewer than 512 of K each, in whole stages.  A function of N and K alone: a row's
+    // sums do not depend on the rows beside it.  (More rows are more rounds of CTAs, each with its start and end, where a
+    // split by the batch made each CTA's range longer: 128 rows x 128 x 110,592 48 -> 66 us, 65 x 256 x 221,184 130 -> 144.)
+    const int mt = (a.N + kM - 1) / kM;
+    const int want = std::max(1, std::min(sms / mt, (a.K + 511) / 512));
     const int kper = ((a.K + want - 1) / want + kBK - 1) / kBK * kBK;
     a.splits = (a.K + kper - 1) / kper;
+    // rows whose partials fit (splits x N is under 128 x sms, or N with one split): a launch takes those
+    size_t rows = std::max<size_t>(1, partials / ((size_t)a.splits * a.N));
+    if (rows >= kN) rows = rows / kN * kN;
     cudaFuncSetAttribute(dense_f32tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    dense_f32tc_kernel<<<dim3(mt, a.splits, bt), kThreads, kSmem, s>>>(a, kper);
-    launch_dense_reduce(a, s);
+    const int total = a.B;
+    for (int b0 = 0; b0 < total; b0 += a.B) {
+        a.B = (int)std::min<size_t>(rows, total - b0);
+        dense_f32tc_kernel<<<dim3(mt, a.splits, (a.B + kN - 1) / kN), kThreads, kSmem, s>>>(a, kper);
+        launch_dense_reduce(a, s);
+        a.x += (size_t)a.B * a.K;
+        a.y += (size_t)a.B * a.N;
+    }
 }
 
 }  // namespace fusion

@@ -6,9 +6,12 @@
 // budget, or a host application whose allocator owns all device memory), or a
 // caller in a latency-bound request loop that cannot afford the implicit
 // device synchronisation and unbounded latency that cudaMalloc / cudaFree may
-// bring.  Such a caller provides its inputs and outputs and gets the same
-// result as the split-K dense layer of fusion_score, with the split partials
-// kept in the static array below instead of a model workspace.
+// bring.  Such a caller provides its inputs and outputs and gets the dense
+// layer of an FP32 model's fusion_score, with the split partials kept in the
+// static array below instead of a model workspace: up to 8 rows by the same
+// kernels with the same bits, above that on the tensor cores at FP32's accuracy
+// (k_dense_f32tc.cu), whose sums are in another order.  On either side of that
+// line a row's result does not depend on the rows beside it or on their number.
 //
 // The scratch array lives in every GPU that loads this library, for the
 // lifetime of the process (8 MiB).  Host code cannot use the array's name as a
@@ -37,6 +40,7 @@ namespace {
 
 std::mutex g_noalloc_mu;
 void *g_scratch_addr[FUSION_NOALLOC_MAX_DEVICES] = {};
+int g_sms[FUSION_NOALLOC_MAX_DEVICES] = {};
 
 int noalloc_fail(int code, const std::string &m) { return fusion::set_last_error(code, m.c_str()); }
 
@@ -64,6 +68,7 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
     if (e != cudaSuccess) return noalloc_fail(FUSION_ECUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
     if (dev < 0 || dev >= FUSION_NOALLOC_MAX_DEVICES) return noalloc_fail(FUSION_EINVAL, "device index too large");
     void *scratch = nullptr;
+    int sms = 0;
     {
         std::lock_guard<std::mutex> lock(g_noalloc_mu);
         if (!g_scratch_addr[dev]) {
@@ -71,9 +76,13 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
             e = cudaGetSymbolAddress(&p, g_dense_scratch);
             if (e != cudaSuccess)
                 return noalloc_fail(FUSION_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
+            e = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+            if (e != cudaSuccess)
+                return noalloc_fail(FUSION_ECUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
             g_scratch_addr[dev] = p;
         }
         scratch = g_scratch_addr[dev];
+        sms = g_sms[dev];
     }
     // an error left pending by earlier work would otherwise be reported below as this call's launch failure
     e = cudaPeekAtLastError();
@@ -84,10 +93,8 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
     // up to 8 rows the weight stream bounds either form and the CUDA-core one has less to set up; above that its
     // multiply-adds do (us, CUDA cores / tensor cores: 256 x 221,184 59 / 66 at 8 rows and 88 / 67 at 16, 64 x 16,000
     // 18.5 / 20.5 and 26 / 20.5)
-    if (B > 8) {
-        a.splits = (int)(FUSION_NOALLOC_MAX_PARTIALS / ((long long)B * N));     // the scratch's room, at least `splits`
-        fusion::launch_dense_f32tc(a, static_cast<cudaStream_t>(cuda_stream));
-    } else fusion::launch_dense(a, static_cast<cudaStream_t>(cuda_stream));
+    if (B > 8) fusion::launch_dense_f32tc(a, FUSION_NOALLOC_MAX_PARTIALS, sms, static_cast<cudaStream_t>(cuda_stream));
+    else fusion::launch_dense(a, static_cast<cudaStream_t>(cuda_stream));
     e = cudaGetLastError();
     if (e != cudaSuccess) return noalloc_fail(FUSION_ECUDA, std::string("dense launch: ") + cudaGetErrorString(e));
     return FUSION_OK;

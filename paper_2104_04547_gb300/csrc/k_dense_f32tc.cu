@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
     const int n0 = blockIdx.x * kM, b0 = blockIdx.z * kN;
     const int kbeg = blockIdx.y * kper, kend = min(a.K, kbeg + kper);
     const int iters = (kend - kbeg + kBK - 1) / kBK;
-    const uint64_t deadline = tc::globaltimer() + kWaitNs;
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&full[i], kConv); tc::mbar_init(&empty[i], 1); }
         tc::mbar_init(done, 1);
@@ -87,6 +86,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f32tc_kernel(DenseArgs a, i
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tbase = *tmem_slot;
+    const uint64_t deadline = tc::globaltimer() + kWaitNs;     // once the tensor memory is held: another kernel may have had it
     const int sums = (iters + kSumIters - 1) / kSumIters;
 
     if (warp < kConvWarps) {

@@ -128,7 +128,6 @@ __global__ void __launch_bounds__(kThreads, 1) sg_gru_tc_kernel(SgGruTcArgs a) {
     if (A > a.A) A = a.A;
     const int n_tiles = (A + kTileM - 1) / kTileM;
     const bool any_T = a.T_out[0] || a.T_out[1];
-    const uint64_t deadline = tc::globaltimer() + kWaitNs;
 
     if (tid == 0) {
         tc::mbar_init(w_bar, 1);
@@ -170,6 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_gru_tc_kernel(SgGruTcArgs a) {
     }
 
     wait_prior();            // the weights (this kernel's own) are on their way; what follows reads the step before
+    const uint64_t deadline = tc::globaltimer() + kWaitNs;     // the time spent waiting for earlier kernels does not count
     const uint32_t s0 = tc::smem_u32(smem);
     const uint32_t sMhi = s0 + P::oMhi, sMlo = s0 + P::oMlo, sHhi = s0 + P::oHhi, sHlo = s0 + P::oHlo;
     const int quarter = warp & 3;
@@ -380,7 +380,6 @@ __global__ void __launch_bounds__(kThreads, 1) sg_stage_tc_kernel(SgStageTcArgs 
     const int n_tiles = (A + kTileM - 1) / kTileM;
     const bool gate = a.wg != nullptr && a.h_in != nullptr;
     const bool any_T = a.T_out[0] || a.T_out[1];
-    const uint64_t deadline = tc::globaltimer() + kWaitNs;
 
     if (tid == 0) {
         tc::mbar_init(w_bar, 1);
@@ -417,6 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) sg_stage_tc_kernel(SgStageTcArgs 
     }
 
     wait_prior();            // the weights (this kernel's own) are on their way; what follows reads the step before
+    const uint64_t deadline = tc::globaltimer() + kWaitNs;     // the time spent waiting for earlier kernels does not count
     const uint32_t s0 = tc::smem_u32(smem);
     const uint32_t sXhi = s0 + P::oXhi, sXlo = s0 + P::oXlo, sYhi = s0 + P::oYhi, sYlo = s0 + P::oYlo;
     const int quarter = warp & 3;

@@ -218,8 +218,9 @@ int fusion_last_timings(fusion_model *m, float *out, int32_t n);
                                             call the first tensor-core conv launch loads nothing, so its
                                             bounded waits run out (about 1 s): the call returns
                                             FUSION_ETIMEOUT with the output untouched, and later calls are
-                                            normal.  Nothing faults or hangs.  FUSION_EUNSUPPORTED on the
-                                            FP32 path or with CUDA graphs on.  Value 2: the same for the
+                                            normal.  Nothing faults or hangs.  FUSION_EUNSUPPORTED for an
+                                            FP32 model with every layer on the CUDA cores, or with CUDA graphs
+                                            on.  Value 2: the same for the
                                             first tensor-core graph launch (its weight copy is not issued);
                                             FUSION_EUNSUPPORTED unless the graph runs on the tensor cores */
 

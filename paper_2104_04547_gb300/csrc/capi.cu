@@ -1631,8 +1631,10 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value) {
         if (value != 1 && value != 2) return fail(FUSION_EINVAL, "the wait-timeout test takes value 1 or 2");
         if (m->use_graph) return fail(FUSION_EUNSUPPORTED, "turn CUDA graphs off for the wait-timeout test");
         if (value == 1) {
-            if (!m->bf16) return fail(FUSION_EUNSUPPORTED, "the conv wait-timeout test needs a BF16 or FP8 model");
-            conv_tc_stall_next(m->tcplan[0]);
+            const int i = (int)(std::find(m->f32tc, m->f32tc + m->d.n_conv, true) - m->f32tc);
+            if (m->bf16) conv_tc_stall_next(m->tcplan[0]);
+            else if (i < m->d.n_conv) conv_f32tc_stall_next(m->f32plan[i]);
+            else return fail(FUSION_EUNSUPPORTED, "the model has no convolution on the tensor cores");
         } else {
             if (!m->sg_tc) return fail(FUSION_EUNSUPPORTED, "the graph convolution is not on the tensor cores");
             m->sg_stall_next = true;

@@ -264,7 +264,9 @@ struct ConvF32TcSpec {
 int conv_f32tc_plan(ConvF32TcPlan &plan, const ConvF32TcSpec &spec, char *why, size_t why_len);
 // Poses p0 .. p0 + B - 1 of the call, whose parts are the buffer's poses 0 .. B - 1.  amax: their max |output|, infinities
 // aside (atomic max, zeroed by the caller), or null.  Returns the tile.
-ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s);
+ConvTile conv_f32tc_launch(ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s);
+// As conv_tc_stall_next.
+void conv_f32tc_stall_next(ConvF32TcPlan &plan);
 // Output channels per tile (0: c_out is not a multiple of 32).
 int conv_f32tc_block(int c_out);
 // Weights in two FP16 parts, w * s_w[co] = hi + lo with s_w a power of two (of the channel's finite weights; an infinite

@@ -93,6 +93,7 @@ struct Args {
     int blocked;           // input layout: 0 NDHWC, 1 channel-blocked, 2 parity-split
     Geo g;
     unsigned *err;
+    int stall;             // test of the bounded waits: the producer loads nothing
     int *tile_counter;     // [0] tiles handed out beyond each CTA's first, [1] CTAs done (both zero between launches)
 };
 
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
             const bool done = tile >= n_tiles || *abort_flag;
             tile_ring[slot] = done ? -1 : tile;
             tc::mbar_arrive(&tile_full[slot]);
-            if (done) break;
+            if (done || a.stall) break;
             int x0, y0, z0, c0, b;
             decode(tile, x0, y0, z0, c0, b);
             size_t woff = (size_t)(c0 / NT) * a.wblk;   // stored channel block, chunk, phase, (ty, tx) group
@@ -776,8 +777,10 @@ static void launch_t(const ConvF32TcPlan::Impl &P, const ConvF32TcPlan::Impl::Va
     conv3d_f32tc_kernel<NT, T><<<grid, Roles<NT, T>::THREADS, V.smem, s>>>(V.tmap, a);
 }
 
-ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s) {
-    const ConvF32TcPlan::Impl &P = *plan.impl;
+void conv_f32tc_stall_next(ConvF32TcPlan &plan) { plan.impl->args.stall = 1; }
+
+ConvTile conv_f32tc_launch(ConvF32TcPlan &plan, int p0, int B, float *amax, cudaStream_t s) {
+    ConvF32TcPlan::Impl &P = *plan.impl;
     // the tile with the shortest schedule: rounds of tiles over the SMs x a tile's MMA clocks
     int best = 0;
     double best_t = 1e300;
@@ -797,6 +800,7 @@ ConvTile conv_f32tc_launch(const ConvF32TcPlan &plan, int p0, int B, float *amax
     a.inv_sx += p0;
     a.y += maps;
     if (a.residual) a.xres += maps;
+    P.args.stall = 0;      // one launch only
     switch (P.NT * 16 + V.T) {
     case 32 * 16 + 8: launch_t<32, 8>(P, V, a, s); break;
     case 32 * 16 + 4: launch_t<32, 4>(P, V, a, s); break;

@@ -258,6 +258,13 @@ int fusion_last_timings(fusion_model *m, float *out, int32_t n);
                                              layers and drops captured graphs; FUSION_EUNSUPPORTED on the
                                              FP32 path */
 
+#define FUSION_OPT_TEST_CONV_TILE 8   /* test of the tensor-core convs' tiles (BF16, FP8): value t >= 0 = every layer takes
+                                         tile t of those it chooses from by batch size (0 the planned one, then
+                                         the smaller ones; a layer with fewer its last) in calls of any size; -1 =
+                                         the choice by the estimate.  Scores are the same in every mode.  Drops captured graphs;
+                                         planning anew (other options, the autotuner) ends it.
+                                         FUSION_EUNSUPPORTED on the FP32 path */
+
 /* Set a runtime option of a model (FUSION_OPT_*). */
 int fusion_set_option(fusion_model *m, int32_t option, int64_t value);
 

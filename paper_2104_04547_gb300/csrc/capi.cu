@@ -1692,6 +1692,14 @@ int fusion_set_option(fusion_model *m, int32_t option, int64_t value) {
         drop_graphs(m);
         return FUSION_OK;
     }
+    case FUSION_OPT_TEST_CONV_TILE:
+        if (value < -1 || value > 16) return fail(FUSION_EINVAL, "the conv tile test takes -1 or a tile's index");
+        if (!m->bf16) return fail(FUSION_EUNSUPPORTED, "the FP32 path has no tensor-core tiles");
+        for (int i = 0; i < m->d.n_conv; ++i)
+            if (value < 0) conv_tc_tune(m->tcplan[i], 0, 0);
+            else conv_tc_tune(m->tcplan[i], -1, std::min((int)value, conv_tc_tiles(m->tcplan[i]) - 1));
+        drop_graphs(m);
+        return FUSION_OK;
     default:
         return fail(FUSION_EINVAL, "unknown option");
     }

@@ -46,6 +46,7 @@ FUSION_OPT_GRAPH_NODES_PER_WARP = 4
 FUSION_OPT_SERIAL_BRANCHES = 5
 FUSION_OPT_GRAPH_TENSOR_CORES = 6
 FUSION_OPT_CONV_STRIDE2_SPLIT = 7
+FUSION_OPT_TEST_CONV_TILE = 8
 
 EXPORTED = ["fusion_weights_bytes", "fusion_create", "fusion_score", "fusion_destroy", "fusion_last_error",
             "fusion_stage_bytes", "fusion_fetch_stage", "fusion_last_timings", "fusion_cnn_dense_noalloc",

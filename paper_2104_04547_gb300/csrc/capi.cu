@@ -770,15 +770,22 @@ int alloc_workspace(fusion_model *m) {
 }  // namespace
 
 // Whether a call's kernels start early (launch_kernel), where they leave most multiprocessors idle: at most 48 tiles of 128
-// graph nodes, a third of the multiprocessors (10 paper-size poses).  Paper-final model, host call: one pose 311 -> 255 us,
-// two 372 -> 330, four 446 -> 396 (most of it the graph branch's kernels, see below); from eight on, and for the full-size
-// model, whose tiles fill the chip, the same either way (615 and 614, 628 and 630 us).
+// graph nodes, a third of the multiprocessors (12 poses of 500 atoms).  Host calls without and with it, us: paper-final BF16
+// one pose 300 -> 248, two 369 -> 331, four 466 -> 412 (most of it the graph branch's kernels, see below), five to twelve
+// the same; FP8 one 300 -> 279, four 450 -> 418, eight 585 -> 538, ten 641 -> 638; 20^3 one 182 -> 167, eight 233 -> 218,
+// twelve 250 -> 241; 24^3 FP32 one 207 -> 200, eight 397 -> 394; full-size, whose tiles fill the chip, within 0.5% (628 and
+// 625, 4302 and 4301).  The largest loss seen is 24^3 BF16 at eight poses, 230 -> 234.
 static bool early_launches(int atoms) { return atoms <= 128 * 48; }
 
-// Of those, the calls whose graph branch takes longer than the convolutions it runs beside (one to three poses of the
+// Of those, the calls whose graph branch takes longer than the convolutions it runs beside (one to four poses of the
 // paper-final model, whose nine steps were 60% of the call): there the graph's kernels start early too, and the
 // convolutions' tiles are chosen for the multiprocessors that its waiting CTAs do not hold.  Elsewhere those CTAs would
 // only keep multiprocessors from the convolutions (full-size model, one pose: 627 -> 657 us).
+// A coarse estimate: the branch is a chain of launches whose times hardly depend on the atoms while these fit the chip, so
+// its constants are those of 500 atoms.  Host calls never and by this rule, us, at 224, 480 and 800 atoms a pose: paper-final
+// BF16 one pose 274 -> 235, 305 -> 251, 344 -> 269, four 412 -> 386, 468 -> 415, 531 -> 430; FP8 one 270 -> 257, 303 -> 278,
+// 350 -> 302; 20^3 BF16 one 162 -> 155, 182 -> 159, 213 -> 181; 24^3 BF16 one 144 -> 137, 162 -> 147, 196 -> 172; full-size
+// the same.
 constexpr int kGraphSms = 24;       // 16 CTAs of messages and 5 of GRU tiles for 500 atoms
 static bool graph_is_longer(const fusion_model *m, int B) {
     if (!m->sg_tc || !m->bf16) return false;

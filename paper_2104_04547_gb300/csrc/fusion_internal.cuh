@@ -202,7 +202,7 @@ struct ConvTcSpec {
     unsigned *err;
     int T;                  // output slices per CTA (0: default for c_out)
     int alts;               // also plan smaller tiles, for conv_tc_launch to choose from by batch size
-    int groups_per_stage;   // (ty, tx) kernel-offset groups per weight stage (0: about 48 KB per stage)
+    int groups_per_stage;   // (ty, tx) kernel-offset groups per weight stage (0: about 56 KB per stage, 72 KB at stride 2)
     int nbs;                // weight stages in the ring (0: 2)
     int group;              // output slices per MMA (1, 2, 4; N = group x c_out); <= 0: default for the layer
     int fold;               // x-folded first-layer input: 0 no, 1 bf16 grid (VoxArgs::fold_pad = k / 2),

@@ -1087,10 +1087,9 @@ static int plan_tile(ConvTcPlan::Impl &P, const ConvTcSpec &sp, bool alt, char *
     g.stage_bytes = ((uint32_t)g.groups_per_stage * gbytes_max + 127) / 128 * 128;
     // output slices per MMA: by default the most (4, else 2) that fit, for stride 1.  Measured on the
     // 64-channel layers (64 poses, BF16, persistent kernel): 2 slices 10.4-10.5 ms, 4 slices 10.1-10.3 ms per
-    // residual layer.  (Before the epilogue had warps of its own, 4 lost to 2: one thread issues an MMA
-    // about every 80-100 clocks, and 4 slices per MMA leave two accumulator sets, hence two issuers, whose
-    // warps also ran the epilogue.)  At stride 2 each phase has only 2-3 z offsets, so a slice group
-    // shares little: 1.
+    // residual layer, with MMAs issued every 166 to 210 clocks by a warp; they now take 45 (issue_groups), which
+    // four slices per MMA need least.  At stride 2 each phase has only 2-3 z offsets, so a slice group shares
+    // little: 1.
     auto group_ok = [&](int G) {
         return (G == 1 || G == 2 || G == 4 || G == 8) && T % G == 0 && G * c_out <= 256 && T / G >= (G == 8 ? 2 : 1);
     };

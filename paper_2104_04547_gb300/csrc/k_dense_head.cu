@@ -13,9 +13,9 @@
 //     k-quads of rows as they lie in memory (a transpose would cost as many stores as the loads it saves).
 // The line between them is where 16 sums per weight still fit a lane and cost less than the stream (23 of 33 us).
 // The weight rows were permuted at model creation so that the flatten of the NDHWC pooled map is a plain row read.
-// Measured with the reduction, through the no-allocation entry: 4 x 128 x 110,592 127 -> 21.5 us (58 MB, 2.7 TB/s),
-// 64 x 256 x 221,184 266 -> 197 us (36.8 TFLOP/s); the dense layer of the single-pose 24^3 model 100 -> 16 us, of the
-// full-size model at 3 poses 256 -> 61 us.  Errors against float64 fell from 6e-7 to 2.4e-7 (chains of 256, not 2048).
+// Measured with the reduction: 4 x 128 x 110,592 127 -> 21.5 us (58 MB, 2.7 TB/s; through the no-allocation entry, which
+// takes these kernels up to 8 rows), 64 x 256 x 221,184 266 -> 197 us (36.8 TFLOP/s); the dense layer of the single-pose
+// 24^3 model 100 -> 16 us, of the full-size model at 3 poses 256 -> 61 us.  Errors against float64 fell from 6e-7 to 2.4e-7 (chains of 256, not 2048).
 //
 // Fusion head (Section 3.3.3, Table V: fusion dense layers with SELU): one CTA
 // per pose runs Linear -> SELU -> ... -> Linear on [cnn latent, sg latent].

@@ -91,8 +91,10 @@ extern "C" int fusion_cnn_dense_noalloc(const float *x, const float *w, const fl
                                               cudaGetErrorString(e));
     fusion::DenseArgs a{x, w, bias, static_cast<float *>(scratch), y, B, N, K, splits, relu ? 1 : 0, false};
     // up to 8 rows the weight stream bounds either form and the CUDA-core one has less to set up; above that its
-    // multiply-adds do (us, CUDA cores / tensor cores: 256 x 221,184 59 / 66 at 8 rows and 88 / 67 at 16, 64 x 16,000
-    // 18.5 / 20.5 and 26 / 20.5)
+    // multiply-adds do.  us, CUDA cores / tensor cores, at 8 rows (the tensor-core figure is that of 9) and at 12:
+    //   24 x 110,592   21 / 27, 27 / 27      64 x 16,000   21 / 23, 28 / 23     128 x 16,000   21 / 23, 29 / 23
+    //   128 x 110,592  29 / 29, 37 / 29     300 x 16,000   21 / 23, 29 / 23    300 x 110,592   48 / 58, 64 / 58
+    //   256 x 221,184  68 / 72, 91 / 72
     if (B > 8) fusion::launch_dense_f32tc(a, FUSION_NOALLOC_MAX_PARTIALS, sms, static_cast<cudaStream_t>(cuda_stream));
     else fusion::launch_dense(a, static_cast<cudaStream_t>(cuda_stream));
     e = cudaGetLastError();

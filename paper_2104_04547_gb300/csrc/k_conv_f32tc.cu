@@ -158,10 +158,6 @@ __device__ __forceinline__ void issue_nz(int nz, uint32_t on, uint32_t dt, uint3
     }
 }
 
-// t / (s_w s_x) from the inverse scales, powers of two from 2^-126 to 2^113: the smaller one first, so that no step
-// overflows, or goes below the normal range, where the result does not.
-__device__ __forceinline__ float unscale(float t, float isw, float isx) { return t * fminf(isw, isx) * fmaxf(isw, isx); }
-
 template <int NT, int T>
 __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                 Args a) {
@@ -462,7 +458,9 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
             int x0, y0, z0, c0, b;
             decode(tile, x0, y0, z0, c0, b);
             const int n = a.n_out, yy = y0 + h, xx = x0 + w;
-            const float isx = a.inv_sx[b];
+            // 1 / s_x, a power of two as 1 / s_w is: before 1 / s_w where it is below 1 and after it elsewhere, so that no step
+            // overflows, or goes below the normal range, where the result does not
+            const float isx = a.inv_sx[b], sx_lo = fminf(isx, 1.f), sx_hi = fmaxf(isx, 1.f);
             float vmax = 0.f;
 #pragma unroll
             for (int o = 0; o < OWN; ++o) {
@@ -475,19 +473,28 @@ __global__ void __launch_bounds__(Roles<NT, T>::THREADS, 1) conv3d_f32tc_kernel(
                     const float4 bs = __ldg(reinterpret_cast<const float4 *>(a.bias + c0) + j4);
                     const float *t = tot[o] + j4 * 4;
                     float4 v;
-                    v.x = fmaxf(unscale(t[0], sw.x, isx) + bs.x, 0.f);
-                    v.y = fmaxf(unscale(t[1], sw.y, isx) + bs.y, 0.f);
-                    v.z = fmaxf(unscale(t[2], sw.z, isx) + bs.z, 0.f);
-                    v.w = fmaxf(unscale(t[3], sw.w, isx) + bs.w, 0.f);
+                    v.x = fmaxf(t[0] * sx_lo * sw.x * sx_hi + bs.x, 0.f);
+                    v.y = fmaxf(t[1] * sx_lo * sw.y * sx_hi + bs.y, 0.f);
+                    v.z = fmaxf(t[2] * sx_lo * sw.z * sx_hi + bs.z, 0.f);
+                    v.w = fmaxf(t[3] * sx_lo * sw.w * sx_hi + bs.w, 0.f);
                     if (a.residual) {
                         const float4 x4 = __ldg(reinterpret_cast<const float4 *>(a.xres + at) + j4);
                         v.x += x4.x; v.y += x4.y; v.z += x4.z; v.w += x4.w;
                     }
-                    vmax = fmaxf(vmax, fmaxf(fmaxf(finite_abs(v.x), finite_abs(v.y)), fmaxf(finite_abs(v.z), finite_abs(v.w))));
+                    vmax = fmaxf(vmax, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
                     reinterpret_cast<float4 *>(a.y + at)[j4] = v;
                 }
             }
             if (a.amax) {
+                if (vmax == INFINITY) {         // rare: the finite ones, from what this thread just stored
+                    vmax = 0.f;
+                    for (int o = 0; o < OWN; ++o) {
+                        const int zz = z0 + e0 + EG * o;
+                        if (zz >= n || yy >= n || xx >= n) continue;
+                        const float *own = a.y + ((((size_t)b * n + zz) * n + yy) * n + xx) * a.c_out + c0;
+                        for (int j = 0; j < NT; ++j) vmax = fmaxf(vmax, finite_abs(own[j]));
+                    }
+                }
                 for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
                 if (lane == 0 && vmax > 0.f) atomicMax(reinterpret_cast<unsigned *>(a.amax + b), __float_as_uint(vmax));
             }

@@ -136,10 +136,18 @@ def launches_per_step(desc, n_poses=64):
     # prep + voxelize, the convs, the pool, dense + its reduction (and a second dense layer's two), the radius
     # graph (count, scan, fill; one launch up to 16 poses),
     # a transform per stage, the steps (tensor-core models: message sums, then the tensor-core GRU), the gather,
-    # the head; FP8 and FP32 models: a pass per conv that makes its input's codes or FP16 parts
+    # the head; FP8 and FP32 models: a pass per conv that makes its input's codes or FP16 parts; FP32: a conv and its
+    # pass for every 512 MB of parts (the largest conv input of a pose, 4 bytes per element)
     per_step = 2 if desc.get("dtype", "f32") != "f32" else 1
-    return (2 + len(desc["conv"]) + (1 if desc["pool"] > 1 else 0) + 2 + (2 if desc.get("cnn_dense2") else 0) +
-            (3 if n_poses > 16 else 1) + (0 if desc.get("dtype") == "bf16" else len(desc["conv"])) +
+    convs = len(desc["conv"]) * (1 if desc.get("dtype") == "bf16" else 2)
+    if desc.get("dtype", "f32") == "f32":
+        n, pose = desc["grid_n"], 0
+        for i, c in enumerate(desc["conv"]):
+            pose = max(pose, 4 * n ** 3 * (32 if i == 0 else c["c_in"]))
+            n = (n + 2 * (c["k"] // 2) - c["k"]) // c["stride"] + 1
+        convs *= -(-n_poses // max(1, (512 << 20) // pose))
+    return (2 + convs + (1 if desc["pool"] > 1 else 0) + 2 + (2 if desc.get("cnn_dense2") else 0) +
+            (3 if n_poses > 16 else 1) +
             len(desc["sg_stages"]) + per_step * sum(s["steps"] for s in desc["sg_stages"]) + 1 + 1)
 
 
